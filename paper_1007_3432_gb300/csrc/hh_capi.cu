@@ -13,6 +13,7 @@
 #include "hh_apply.cuh"
 #include "hh_engine.cuh"
 #include "hh_kernels.cuh"
+#include "hh_onchip.cuh"
 #include "hh_trace.cuh"
 
 using namespace hh;
@@ -31,9 +32,10 @@ struct EngStats {
 };
 
 // New solves: states MODE_NEW, empty signal slots for 'parts' tile partials,
-// iteration counter 0.
+// iteration counter 0; the on-chip engine's phase numbers (seq, may be null)
+// go on from where the last launch ended.
 __global__ void k_engine_reset(EngState *s0, EngState *s1, int nsys, unsigned long long *sig, int parts,
-                               EngCtl *ctl, long long timeout_ns, int drop_sig)
+                               EngCtl *ctl, long long timeout_ns, int drop_sig, unsigned long long *seq)
 {
     for (int s = threadIdx.x; s < nsys; s += blockDim.x) {
         EngState z;
@@ -50,6 +52,7 @@ __global__ void k_engine_reset(EngState *s0, EngState *s1, int nsys, unsigned lo
         ctl->k_end = 0;
         ctl->timeout_ns = timeout_ns;
         ctl->drop_sig = drop_sig;
+        if (seq) seq[0] = seq[1] + 1;
     }
 }
 
@@ -116,6 +119,7 @@ struct Plan {
     const double *b = nullptr;
     double *x = nullptr;
     EngSystem sys[64];           // host copy of the device system table (n_pf <= 64)
+    OcPlan oc;                   // layout of the on-chip engine (ok = 0: the grid engine)
 };
 
 }  // namespace
@@ -147,6 +151,14 @@ struct hh_ctx {
     EngStats *d_stats;
     int max_tiles;
     Plan plan;
+    // On-chip engine: packets of two vectors per system, partial-sum packets,
+    // phase numbers; oc_max_rhs systems at most (0: never used), and the
+    // number of systems the packets were last used for.
+    unsigned char *d_pkt;
+    ulonglong2 *d_slots;
+    unsigned long long *d_seq;
+    int oc_max_rhs, oc_last;
+    int smem_sm, smem_blk;
     EngTotals *d_totals;
     // counters and optional CUDA-event profile of the engine launches
     long long n_launch, n_engine;
@@ -210,11 +222,38 @@ void free_ctx(hh_ctx *c)
     for (double *p : {c->obs_eta, c->obs_rhs, c->obs_y, c->obs_part, c->obs_out})
         if (p) cudaFree(p);
     if (c->L16) cudaFree(c->L16);
+    if (c->d_pkt) cudaFree(c->d_pkt);
+    if (c->d_slots) cudaFree(c->d_slots);
+    if (c->d_seq) cudaFree(c->d_seq);
     if (c->ev) {
         for (int i = 0; i < c->ev_cap; ++i)
             if (c->ev[i]) cudaEventDestroy(c->ev[i]);
         free(c->ev);
     }
+}
+
+// Bytes of the on-chip engine's packets for n_rhs systems: two vectors each.
+size_t oc_packets(const hh_ctx *c, int n_rhs)
+{
+    return 2 * oc_packet_bytes(c->prm.precision != HH_FP64) * (size_t)c->N * (size_t)n_rhs;
+}
+
+// Layout of the on-chip engine for n_rhs systems of this context.
+OcPlan ctx_oc_plan(const hh_ctx *c, int n_rhs)
+{
+    OcPlan none = {};
+    if (c->prm.link_order != 0 || c->l16_mode != 0) return none;
+    // An explicit choice of the grid engine's form is a choice of that engine.
+    for (const char *name : {"HH_ENGINE_SLOTS", "HH_ENGINE_OVERLAP", "HH_ENGINE_CTL_WARPS",
+                             "HH_ENGINE_BLOCKS_PER_SM", "HH_ENGINE_PREFETCH"})
+        if (getenv(name)) return none;
+    if (const char *e = getenv("HH_ENGINE_ONCHIP"))
+        if (atoi(e) == 0) return none;
+    const bool mixed = c->prm.precision != HH_FP64;
+    OcPlan p = oc_plan(c->lat.d, c->lat.nx, c->lat.ntau, n_rhs, mixed, c->prm.cheb_degree > 0, c->nsm,
+                       (size_t)c->smem_sm, (size_t)c->smem_blk);
+    if (p.ok && oc_max_blocks(p, c->lat.d) * c->nsm < p.go * p.gt * n_rhs) p.ok = 0;
+    return p;
 }
 
 // Build (or reuse) the engine plan for n_rhs systems b_a -> x_a.
@@ -306,6 +345,15 @@ int make_plan(hh_ctx *c, const double *b, double *x, int n_rhs)
     P.b = b;
     P.x = x;
     P.precision = c->prm.precision;
+    P.oc.ok = 0;
+    if (n_rhs <= c->oc_max_rhs) {
+        P.oc = ctx_oc_plan(c, n_rhs);
+        // Other tiles publish other sites: forget the packets of the last layout.
+        if (P.oc.ok && c->oc_last != n_rhs) {
+            HH_TRY(cudaMemsetAsync(c->d_pkt, 0, oc_packets(c, c->oc_max_rhs), c->stream));
+            c->oc_last = n_rhs;
+        }
+    }
     return HH_OK;
 }
 
@@ -344,8 +392,37 @@ int run_engine(hh_ctx *c)
     TraceRange tr("hh engine solve");
     const Plan &P = c->plan;
     k_engine_reset<<<1, 256, 0, c->stream>>>(c->d_state[0], c->d_state[1], P.nsys, c->d_sig,
-                                             c->max_tiles, c->d_ctl, c->timeout_ns, engine_drop_signal());
+                                             c->max_tiles, c->d_ctl, c->timeout_ns, engine_drop_signal(),
+                                             c->d_seq);
     HH_TRY(cudaGetLastError());
+    bool rec = c->profile && c->ev_used + 2 <= c->ev_cap;
+    if (rec) HH_TRY(cudaEventRecord(c->ev[c->ev_used], c->stream));
+    // A mixed system that ends in FP64 steps leaves the on-chip engine for the
+    // grid engine, which finds the others done.
+    const bool grid_engine = !P.oc.ok || P.oc.mixed;
+    if (P.oc.ok) {
+        OcLaunch O;
+        O.sys = c->d_sys;
+        O.state[0] = c->d_state[0];
+        O.state[1] = c->d_state[1];
+        O.ctl = c->d_ctl;
+        O.pkt = c->d_pkt;
+        O.slots = c->d_slots;
+        O.seq = c->d_seq;
+        O.sig = c->d_sig;
+        O.sig_stride = c->max_tiles;
+        O.nsys = P.nsys;
+        O.N = c->N;
+        O.go = P.oc.go;
+        O.gt = P.oc.gt;
+        O.so = P.oc.so;
+        O.st = P.oc.st;
+        O.x_global = P.oc.x_global;
+        O.drop = engine_drop_signal();
+        O.max_iters = (2LL * c->prm.cheb_degree + 1) * (3LL * (long long)c->prm.cg_maxit + 64);
+        HH_TRY(oc_launch(O, P.oc, c->lat.d, c->stream));
+        c->n_launch += 1;
+    }
     EngLaunch L;
     L.sys = c->d_sys;
     L.state[0] = c->d_state[0];
@@ -363,9 +440,7 @@ int run_engine(hh_ctx *c)
     L.max_iters = (2LL * c->prm.cheb_degree + 1) * (3LL * (long long)c->prm.cg_maxit + 64);
     L.two_slot = c->two_slot;
     L.homogeneous = P.homogeneous;
-    bool rec = c->profile && c->ev_used + 2 <= c->ev_cap;
-    if (rec) HH_TRY(cudaEventRecord(c->ev[c->ev_used], c->stream));
-    HH_TRY(engine_launch(L, P.grid, ENGINE_BLOCK, c->stream, c->kind));
+    if (grid_engine) HH_TRY(engine_launch(L, P.grid, ENGINE_BLOCK, c->stream, c->kind));
     if (rec) {
         HH_TRY(cudaEventRecord(c->ev[c->ev_used + 1], c->stream));
         c->ev_used += 2;
@@ -373,7 +448,7 @@ int run_engine(hh_ctx *c)
     k_engine_fold<<<1, 32, 0, c->stream>>>(c->d_state[0], c->d_state[1], P.nsys, c->d_ctl,
                                            c->d_stats, c->d_totals);
     HH_TRY(cudaGetLastError());
-    c->n_launch += 3;
+    c->n_launch += grid_engine ? 3 : 2;
     c->n_engine += 1;
     return HH_OK;
 }
@@ -611,17 +686,36 @@ int hh_create(hh_ctx **out, const hh_lattice *lat, const hh_params *p, void *cud
         delete c;
         return e == cudaErrorMemoryAllocation ? HH_ENOMEM : HH_ECUDA;
     }
+    {
+        int dev = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&c->nsm, cudaDevAttrMultiProcessorCount, dev);
+        cudaDeviceGetAttribute(&c->smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+        cudaDeviceGetAttribute(&c->smem_blk, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        if (const char *env = getenv("HH_APPLY_MTM")) c->mtm_path = atoi(env);
+    }
+    // The on-chip engine's packets, for as many systems as fit on the chip.
+    for (int k = c->cap_rhs; k >= 1 && c->oc_max_rhs == 0; --k)
+        if (ctx_oc_plan(c, k).ok) c->oc_max_rhs = k;
+    if (c->oc_max_rhs > 0) {
+        const size_t pb = oc_packets(c, c->oc_max_rhs);
+        const size_t sb = sizeof(ulonglong2) * 2 * kOcReplicas * kOcMaxTiles * (size_t)c->oc_max_rhs;
+        e = dalloc(&c->d_pkt, pb);
+        if (e == cudaSuccess) e = cudaMalloc((void **)&c->d_slots, sb);
+        if (e == cudaSuccess) e = dalloc(&c->d_seq, 2);
+        if (e == cudaSuccess) e = cudaMemsetAsync(c->d_slots, 0, sb, c->stream);
+        if (e == cudaSuccess) e = cudaMemsetAsync(c->d_seq, 0, 2 * sizeof(unsigned long long), c->stream);
+        if (e != cudaSuccess) {
+            free_ctx(c);
+            delete c;
+            return e == cudaErrorMemoryAllocation ? HH_ENOMEM : HH_ECUDA;
+        }
+    }
     e = cudaMemsetAsync(c->sigma, 0, n * sizeof(double), c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_ctl, 0, sizeof(EngCtl), c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_sc, 0, sizeof(HmcScalars), c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_totals, 0, sizeof(EngTotals), c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_apply_err, 0, sizeof(int), c->stream);
-    {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&c->nsm, cudaDevAttrMultiProcessorCount, dev);
-        if (const char *env = getenv("HH_APPLY_MTM")) c->mtm_path = atoi(env);
-    }
     if (e == cudaSuccess && p->precision >= HH_MIXED_BF16LINK) {
         c->l16_mode = p->precision == HH_MIXED_BF16LINK ? 1 : 2;
         int ex = 14;

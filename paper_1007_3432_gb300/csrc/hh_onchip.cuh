@@ -1,0 +1,63 @@
+// On-chip CG engine: host/device shared declarations.
+//
+// For lattices whose CG vectors fit in the shared memory of the GPU's SMs,
+// one launch keeps them there for the whole solve.  Every right-hand side is
+// a system of its own, cut into go x gt tiles over (o, tau), o being x for
+// d = 1 and z for d = 3 (a d = 3 tile holds whole x-y planes); one block owns
+// one tile.  What a block needs of its neighbours' tiles (two o columns and
+// one row of slices) and the partial sums travel through global memory in
+// packets that carry their own phase number: a reader polls the packet
+// itself, so neither a fence nor a barrier stands between a value and its use.
+#pragma once
+
+#include "hh_engine.cuh"
+
+namespace hh {
+
+constexpr int kOcMaxThreads = 512;
+
+// How a solve of nsys systems of one lattice is laid out on the chip.
+struct OcPlan {
+    int ok;             // 0: the systems do not fit; use the grid engine
+    int go, gt;         // tiles over o and tau
+    int so, st;         // extents of the largest tile
+    int threads;
+    int x_global;       // x stays in global memory (read and written by its owner only)
+    int mixed, cheb;
+    size_t smem;        // dynamic shared memory per block
+};
+
+struct OcLaunch {
+    const EngSystem *sys;
+    EngState *state[2];
+    EngCtl *ctl;
+    unsigned char *pkt;             // per system: N packets of the vector M reads, N of t = M v
+    ulonglong2 *slots;              // per system, replica and parity: one partial-sum packet per tile
+    unsigned long long *seq;        // [0] last phase number of the launches before this one,
+                                    // [1] of this one (see k_engine_reset)
+    unsigned long long *sig;        // the grid engine's signal slots (hand-over of a mixed system)
+    int sig_stride;
+    int nsys, N;
+    int go, gt, so, st;
+    int x_global;
+    int drop;                       // fault injection: tile (drop - 1) of system 0 never publishes
+                                    // its partial sums; 0: none
+    long long max_iters;
+};
+
+// Packet bytes per site and vector, and partial-sum packets per system.
+inline size_t oc_packet_bytes(bool mixed) { return mixed ? 8 : 16; }
+constexpr int kOcMaxTiles = 608;
+constexpr int kOcReplicas = 8;
+
+// Layout for nsys systems, on nsm SMs with smem_sm bytes of shared memory per
+// SM and smem_blk at most per block.
+OcPlan oc_plan(int d, int nx, int ntau, int nsys, bool mixed, bool cheb, int nsm, size_t smem_sm, size_t smem_blk);
+
+// Blocks of a layout's kernel that one SM holds at once.
+int oc_max_blocks(const OcPlan &P, int d);
+
+// Launches the solve (cooperative: its blocks wait on one another).
+cudaError_t oc_launch(const OcLaunch &L, const OcPlan &P, int d, cudaStream_t st);
+
+}  // namespace hh

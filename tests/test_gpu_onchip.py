@@ -1,0 +1,153 @@
+"""The on-chip CG engine (csrc/hh_onchip.cu): lattices whose vectors stay in
+shared memory for a whole solve, cut into tiles over (x, tau) for d = 1 and
+(z, tau) for d = 3.
+
+Against the oracle's operator (true residual of every solution, 1e-10) and the
+grid engine (HH_ENGINE_ONCHIP=0), which runs the same CG: the two take the same
+steps, so their counts differ by rounding only and their solutions by the
+solver tolerance.  Sizes at the edges of the tiling: tiles of one site or one
+plane, N_x = 2 and N_tau = 2, odd extents that leave uneven tiles, several
+tiles per SM (3 and 4 right-hand sides), the largest that fit.
+"""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+import oracle  # noqa: E402
+import workloads  # noqa: E402
+
+H = workloads.T_HOP * workloads.DTAU
+A = workloads.A_HS
+
+
+@pytest.fixture(scope="module")
+def hh():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1007_3432_gb300 as pkg
+    from paper_1007_3432_gb300 import build
+    build.build()
+    pkg.load()
+    return pkg
+
+
+def dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+def _solve(hh, monkeypatch, onchip, d, nx, ntau, precision, b, sigma, x0=None, **kw):
+    monkeypatch.setenv("HH_ENGINE_ONCHIP", str(onchip))
+    with hh.Context(d, nx, ntau, precision=precision, **kw) as ctx:
+        ctx.set_field(dev(sigma))
+        x = torch.full(b.shape, 3.0, dtype=torch.float64, device="cuda") if x0 is None else dev(x0.copy())
+        ctx.counters_reset()
+        rc, info = ctx.solve(dev(b), x, b.shape[0], guess=x0 is not None, allow=(hh.binding.HH_ENOCONV,))
+        return rc, info, x.cpu().numpy(), ctx.counters()
+
+
+SHAPES = [(1, 2, 2), (1, 2, 7), (1, 3, 2), (1, 17, 5), (1, 33, 40), (1, 300, 11), (1, 731, 24), (3, 2, 2), (3, 2, 9),
+          (3, 3, 5), (3, 5, 16), (3, 8, 20), (3, 13, 10)]
+
+
+@pytest.mark.parametrize("precision,cheb", [("fp64", 0), ("mixed", 0), ("fp64", 4)])
+@pytest.mark.parametrize("d,nx,ntau", SHAPES)
+@pytest.mark.parametrize("n_rhs", [1, 4])
+def test_onchip_solve_matches_oracle_and_grid_engine(hh, monkeypatch, d, nx, ntau, precision, cheb, n_rhs):
+    n = nx ** d * ntau
+    sigma = workloads.sigma_field(n, seed=1500 + nx + ntau)
+    b = np.stack([workloads.source(n, seed=1501, rhs=a) for a in range(n_rhs)])
+    kw = dict(cheb_degree=cheb, cheb_eps=1e-3)
+    rc, info, x, cnt = _solve(hh, monkeypatch, 1, d, nx, ntau, precision, b, sigma, **kw)
+    rc0, info0, x0, cnt0 = _solve(hh, monkeypatch, 0, d, nx, ntau, precision, b, sigma, **kw)
+    assert cnt["kernel_launches"] != cnt0["kernel_launches"] or precision == "fp64"
+    assert rc == 0 and rc0 == 0 and info["converged"] == 1 and info["true_relres"] <= 1e-10
+    lat = oracle.lattice(d, nx, ntau)
+    L = oracle.links(lat, A, sigma)
+    for a in range(n_rhs):
+        res = b[a] - oracle.apply_MTM(lat, H, L, x[a])
+        assert np.linalg.norm(res) <= 1.0001e-10 * np.linalg.norm(b[a])
+    assert abs(info["iterations"] - info0["iterations"]) <= 2 + 0.03 * info0["iterations"], (info, info0)
+    assert np.linalg.norm(x - x0) <= 1e-4 * np.linalg.norm(x0)
+    assert cnt["solves"] == n_rhs and cnt["cg_steps"] > 0
+
+
+@pytest.mark.parametrize("d,nx,ntau,precision,n_rhs", [(3, 16, 64, "fp64", 2), (1, 1024, 160, "fp64", 2),
+                                                       (3, 20, 96, "mixed", 1), (1, 2048, 96, "mixed", 3)])
+def test_onchip_large_lattices(hh, monkeypatch, d, nx, ntau, precision, n_rhs):
+    """Tiles of hundreds to thousands of sites, two and more blocks per SM, x
+    in global memory: capped at 60 steps, where both engines hold the same
+    iterate up to rounding (FP64: 1e-10; FP32 steps between reliable updates:
+    1e-4 of the iterate)."""
+    n = nx ** d * ntau
+    sigma = workloads.sigma_field(n, seed=1600 + nx)
+    b = np.stack([workloads.source(n, seed=1601, rhs=a) for a in range(n_rhs)])
+    rc, info, x, _ = _solve(hh, monkeypatch, 1, d, nx, ntau, precision, b, sigma, cg_maxit=60)
+    rc0, info0, x0, _ = _solve(hh, monkeypatch, 0, d, nx, ntau, precision, b, sigma, cg_maxit=60)
+    assert rc == rc0 == hh.binding.HH_ENOCONV and info["iterations"] == info0["iterations"] == 60
+    tol = 1e-10 if precision == "fp64" else 1e-4
+    assert np.linalg.norm(x - x0) <= tol * np.linalg.norm(x0)
+    assert abs(info["true_relres"] - info0["true_relres"]) <= 1e-3 * info0["true_relres"]
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_onchip_guess_and_zero_source(hh, monkeypatch, precision):
+    d, nx, ntau = 3, 5, 12
+    n = nx ** d * ntau
+    sigma = workloads.sigma_field(n, seed=1700)
+    b = np.stack([workloads.source(n, seed=1701, rhs=a) for a in range(2)])
+    b[1] = 0.0
+    rc, info, x, _ = _solve(hh, monkeypatch, 1, d, nx, ntau, precision, b, sigma)
+    assert rc == 0 and not np.any(x[1]) and info["true_relres"] <= 1e-10
+    x0 = x * (1.0 + 1e-6)
+    x0[1] = 5.0                      # dropped: b = 0 has the solution 0
+    rc2, info2, x2, _ = _solve(hh, monkeypatch, 1, d, nx, ntau, precision, b, sigma, x0=x0)
+    assert rc2 == 0 and not np.any(x2[1]) and info2["true_relres"] <= 1e-10
+    assert info2["iterations"] < info["iterations"]
+    assert np.linalg.norm(x2[0] - x[0]) <= 1e-4 * np.linalg.norm(x[0])
+
+
+@pytest.mark.parametrize("d,nx,ntau", [(1, 48, 64), (3, 6, 16)])
+def test_onchip_mixed_hands_over_to_fp64_steps(hh, monkeypatch, d, nx, ntau):
+    """With reliable_delta = 0.9 each reliable update follows a drop of 10%,
+    which counts as a stall: after two the systems go on with FP64 steps, in
+    the grid engine, from the on-chip state."""
+    n = nx ** d * ntau
+    sigma = workloads.sigma_field(n, seed=1800)
+    b = np.stack([workloads.source(n, seed=1801, rhs=a) for a in range(2)])
+    b[1] = 0.0                       # done on the chip; the other goes on
+    rc, info, x, cnt = _solve(hh, monkeypatch, 1, d, nx, ntau, "mixed", b, sigma, reliable_delta=0.9)
+    rc0, info0, x0, cnt0 = _solve(hh, monkeypatch, 0, d, nx, ntau, "mixed", b, sigma, reliable_delta=0.9)
+    assert cnt["fp64_steps"] > 0 and cnt0["fp64_steps"] > 0, (cnt, cnt0)
+    assert abs(cnt["cg_steps"] - cnt0["cg_steps"]) <= 2 + 0.03 * cnt0["cg_steps"]
+    assert rc == 0 and info["converged"] == 1 and info["true_relres"] <= 1e-10 and not np.any(x[1])
+    lat = oracle.lattice(d, nx, ntau)
+    L = oracle.links(lat, A, sigma)
+    res = b[0] - oracle.apply_MTM(lat, H, L, x[0])
+    assert np.linalg.norm(res) <= 1.0001e-10 * np.linalg.norm(b[0])
+
+
+def test_onchip_layouts_alternate_in_one_context(hh, monkeypatch):
+    """Solves with 1, 3 and 2 right-hand sides in turn (other tiles each) and
+    a repeat give, bit for bit, what a fresh context gives."""
+    monkeypatch.setenv("HH_ENGINE_ONCHIP", "1")
+    d, nx, ntau = 1, 61, 40
+    n = nx * ntau
+    sigma = dev(workloads.sigma_field(n, seed=1900))
+    b = dev(np.stack([workloads.source(n, seed=1901, rhs=a) for a in range(3)]))
+
+    def one(ctx, k):
+        x = torch.zeros(k, n, dtype=torch.float64, device="cuda")
+        ctx.solve(b[:k].clone(), x, k)
+        return x.cpu()
+
+    fresh = {}
+    for k in (1, 2, 3):
+        with hh.Context(d, nx, ntau) as ctx:
+            ctx.set_field(sigma)
+            fresh[k] = one(ctx, k)
+    with hh.Context(d, nx, ntau) as ctx:
+        ctx.set_field(sigma)
+        for k in (1, 3, 2, 1, 1, 3):
+            assert torch.equal(one(ctx, k), fresh[k])
