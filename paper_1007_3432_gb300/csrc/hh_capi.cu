@@ -151,13 +151,17 @@ struct hh_ctx {
     EngStats *d_stats;
     int max_tiles;
     Plan plan;
-    // On-chip engine: packets of two vectors per system, partial-sum packets,
-    // phase numbers; oc_max_rhs systems at most (0: never used), and the
-    // number of systems the packets were last used for.
+    // On-chip engine: one block of device memory, allocated by the first plan that
+    // uses it: partial-sum packets, phase numbers, packets of two vectors per
+    // system (for oc_cap systems), and the number of systems the packets were last
+    // used for.
     unsigned char *d_pkt;
     ulonglong2 *d_slots;
     unsigned long long *d_seq;
-    int oc_max_rhs, oc_last;
+    int oc_cap, oc_last;
+    int oc_forms;           // on-chip engine: 0 not used, 1 by rule, 2 tile form, 3 column form only
+    bool oc_known[65];      // layouts by number of systems (n_pf <= 64), once computed
+    OcPlan oc_plans[65];
     int smem_sm, smem_blk;
     EngTotals *d_totals;
     // counters and optional CUDA-event profile of the engine launches
@@ -222,9 +226,7 @@ void free_ctx(hh_ctx *c)
     for (double *p : {c->obs_eta, c->obs_rhs, c->obs_y, c->obs_part, c->obs_out})
         if (p) cudaFree(p);
     if (c->L16) cudaFree(c->L16);
-    if (c->d_pkt) cudaFree(c->d_pkt);
-    if (c->d_slots) cudaFree(c->d_slots);
-    if (c->d_seq) cudaFree(c->d_seq);
+    if (c->d_slots) cudaFree(c->d_slots);    // d_seq and d_pkt lie behind it
     if (c->ev) {
         for (int i = 0; i < c->ev_cap; ++i)
             if (c->ev[i]) cudaEventDestroy(c->ev[i]);
@@ -238,21 +240,54 @@ size_t oc_packets(const hh_ctx *c, int n_rhs)
     return 2 * oc_packet_bytes(c->prm.precision != HH_FP64) * (size_t)c->N * (size_t)n_rhs;
 }
 
-// Layout of the on-chip engine for n_rhs systems of this context.
-OcPlan ctx_oc_plan(const hh_ctx *c, int n_rhs)
+// The forms of the on-chip engine a context uses (decided when it is created).
+int oc_allowed(const hh_ctx *c)
 {
-    OcPlan none = {};
-    if (c->prm.link_order != 0 || c->l16_mode != 0) return none;
+    if (c->prm.link_order != 0 || c->l16_mode != 0) return 0;
     // An explicit choice of the grid engine's form is a choice of that engine.
     for (const char *name : {"HH_ENGINE_SLOTS", "HH_ENGINE_OVERLAP", "HH_ENGINE_CTL_WARPS",
                              "HH_ENGINE_BLOCKS_PER_SM", "HH_ENGINE_PREFETCH"})
-        if (getenv(name)) return none;
-    if (const char *e = getenv("HH_ENGINE_ONCHIP"))
-        if (atoi(e) == 0) return none;
-    const bool mixed = c->prm.precision != HH_FP64;
-    OcPlan p = oc_plan(c->lat.d, c->lat.nx, c->lat.ntau, n_rhs, mixed, c->prm.cheb_degree > 0, c->nsm,
-                       (size_t)c->smem_sm, (size_t)c->smem_blk);
-    if (p.ok && oc_max_blocks(p, c->lat.d) * c->nsm < p.go * p.gt * n_rhs) p.ok = 0;
+        if (getenv(name)) return 0;
+    const char *e = getenv("HH_ENGINE_ONCHIP");
+    return e ? atoi(e) : 1;
+}
+
+// Layout of the on-chip engine for n_rhs systems, with its device memory; ok = 0:
+// the grid engine solves them.
+OcPlan ctx_oc_plan(hh_ctx *c, int n_rhs)
+{
+    OcPlan none = {};
+    if (c->oc_forms <= 0) return none;
+    if (!c->oc_known[n_rhs]) {
+        const bool mixed = c->prm.precision != HH_FP64;
+        c->oc_plans[n_rhs] = oc_plan(c->lat.d, c->lat.nx, c->lat.ntau, n_rhs, mixed, c->prm.cheb_degree > 0, c->nsm,
+                                     (size_t)c->smem_sm, (size_t)c->smem_blk, c->oc_forms);
+        c->oc_known[n_rhs] = true;
+    }
+    const OcPlan &p = c->oc_plans[n_rhs];
+    if (!p.ok) return none;
+    if (n_rhs > c->oc_cap) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return none;
+        const size_t sb = sizeof(ulonglong2) * 2 * kOcReplicas * kOcMaxTiles * (size_t)n_rhs;
+        unsigned char *blk = nullptr;
+        if (cudaMalloc((void **)&blk, sb + 256 + oc_packets(c, n_rhs)) != cudaSuccess) {
+            cudaGetLastError();
+            return none;
+        }
+        if (c->d_slots) cudaFree(c->d_slots);    // waits for the work that uses it
+        c->d_slots = (ulonglong2 *)blk;
+        c->d_seq = (unsigned long long *)(blk + sb);
+        c->d_pkt = blk + sb + 256;
+        c->oc_cap = n_rhs;
+        c->oc_last = 0;
+        if (cudaMemsetAsync(blk, 0, sb + 256, c->stream) != cudaSuccess) return none;
+    }
+    // Other tiles publish other sites: forget the packets of the last layout.
+    if (c->oc_last != n_rhs) {
+        if (cudaMemsetAsync(c->d_pkt, 0, oc_packets(c, c->oc_cap), c->stream) != cudaSuccess) return none;
+        c->oc_last = n_rhs;
+    }
     return p;
 }
 
@@ -345,15 +380,7 @@ int make_plan(hh_ctx *c, const double *b, double *x, int n_rhs)
     P.b = b;
     P.x = x;
     P.precision = c->prm.precision;
-    P.oc.ok = 0;
-    if (n_rhs <= c->oc_max_rhs) {
-        P.oc = ctx_oc_plan(c, n_rhs);
-        // Other tiles publish other sites: forget the packets of the last layout.
-        if (P.oc.ok && c->oc_last != n_rhs) {
-            HH_TRY(cudaMemsetAsync(c->d_pkt, 0, oc_packets(c, c->oc_max_rhs), c->stream));
-            c->oc_last = n_rhs;
-        }
-    }
+    P.oc = ctx_oc_plan(c, n_rhs);
     return HH_OK;
 }
 
@@ -694,23 +721,6 @@ int hh_create(hh_ctx **out, const hh_lattice *lat, const hh_params *p, void *cud
         cudaDeviceGetAttribute(&c->smem_blk, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
         if (const char *env = getenv("HH_APPLY_MTM")) c->mtm_path = atoi(env);
     }
-    // The on-chip engine's packets, for as many systems as fit on the chip.
-    for (int k = c->cap_rhs; k >= 1 && c->oc_max_rhs == 0; --k)
-        if (ctx_oc_plan(c, k).ok) c->oc_max_rhs = k;
-    if (c->oc_max_rhs > 0) {
-        const size_t pb = oc_packets(c, c->oc_max_rhs);
-        const size_t sb = sizeof(ulonglong2) * 2 * kOcReplicas * kOcMaxTiles * (size_t)c->oc_max_rhs;
-        e = dalloc(&c->d_pkt, pb);
-        if (e == cudaSuccess) e = cudaMalloc((void **)&c->d_slots, sb);
-        if (e == cudaSuccess) e = dalloc(&c->d_seq, 2);
-        if (e == cudaSuccess) e = cudaMemsetAsync(c->d_slots, 0, sb, c->stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(c->d_seq, 0, 2 * sizeof(unsigned long long), c->stream);
-        if (e != cudaSuccess) {
-            free_ctx(c);
-            delete c;
-            return e == cudaErrorMemoryAllocation ? HH_ENOMEM : HH_ECUDA;
-        }
-    }
     e = cudaMemsetAsync(c->sigma, 0, n * sizeof(double), c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_ctl, 0, sizeof(EngCtl), c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_sc, 0, sizeof(HmcScalars), c->stream);
@@ -723,6 +733,7 @@ int hh_create(hh_ctx **out, const hh_lattice *lat, const hh_params *p, void *cud
         c->l16_scale = ldexp(1.0, -ex);
         e = dalloc(&c->L16, n);
     }
+    c->oc_forms = oc_allowed(c);
     if (e == cudaSuccess) e = launch_links(c->geo, p->A, c->sigma, c->L64, c->L32, c->stream);
     if (e == cudaSuccess) e = links16_after(c);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);

@@ -27,269 +27,22 @@
 //
 // What bounds it: the chain exchange - barrier - phase - block sum, run by a few
 // warps (FP64 from about 800 sites per SM: the FP64 pipe, 16 clocks per warp
-// instruction).  Measured against the grid engine, us per iteration, 2
-// right-hand sides: d = 1 32 x 64 FP64 5.9 (11.3), 1024 x 128 FP64 11.4 (15.4),
-// mixed 7.3 (10.7); d = 3 8^3 x 40 FP64 7.7 (17.2), 12^3 x 64 mixed 7.9 (15.0),
-// 16^3 x 64 mixed 9.7 (16.6); a degree-8 preconditioned step on 256 x 256 91 (199).
-// It was faster wherever the vectors fit (20^3 x 64 mixed: 15.9 against 19.4).
+// instruction).  Measured against the grid engine, us per iteration: d = 1
+// 1024 x 128 FP64, 2 right-hand sides, 10.5 (15.4), a degree-8 preconditioned
+// step on 256 x 256 91 (199); d = 3 16^3 x 64 mixed, one, 8.2 (15.1), two, 8.5
+// (16.5), 20^3 x 96 mixed, one, 11.3 (18.2).  It was faster wherever the vectors
+// fit (20^3 x 64 mixed, two: 15.1 against 19.4).  Tiles whose column fits a
+// thread's registers run in hh_onchip_cols.cu.
 //
 // Every wait is bounded (EngCtl::timeout_ns); on expiry the block records
 // HH_ETIMEOUT, and all its threads leave at the next block barrier.
-#include <cstdlib>
+#include <atomic>
 
-#include "hh_engine_decide.cuh"
-#include "hh_onchip.cuh"
+#include "hh_onchip_dev.cuh"
 
 namespace hh {
 
 namespace {
-
-// ---------------------------------------------------------------------------
-// Packets.
-// ---------------------------------------------------------------------------
-struct Raw16 {
-    unsigned long long v, seq;
-};
-
-__device__ __forceinline__ Raw16 ld_raw(const Raw16 *p)
-{
-    Raw16 r;
-    asm volatile("{\n\t.reg .b128 t;\n\tld.relaxed.gpu.global.b128 t, [%2];\n\tmov.b128 {%0, %1}, t;\n\t}"
-                 : "=l"(r.v), "=l"(r.seq)
-                 : "l"(p)
-                 : "memory");
-    return r;
-}
-
-__device__ __forceinline__ void st_raw(Raw16 *p, unsigned long long v, unsigned long long seq)
-{
-    asm volatile("{\n\t.reg .b128 t;\n\tmov.b128 t, {%1, %2};\n\tst.relaxed.gpu.global.b128 [%0], t;\n\t}" ::"l"(p),
-                 "l"(v), "l"(seq)
-                 : "memory");
-}
-
-// One site's packet in a buffer of packets indexed by site.
-template <typename T>
-struct Packet;
-
-template <>
-struct Packet<double> {
-    using Raw = Raw16;
-    static __device__ __forceinline__ Raw load(const unsigned char *buf, int site)
-    {
-        return ld_raw((const Raw16 *)buf + site);
-    }
-    static __device__ __forceinline__ bool ready(const Raw &r, uint32_t seq) { return (uint32_t)r.seq == seq; }
-    static __device__ __forceinline__ double value(const Raw &r) { return __longlong_as_double((long long)r.v); }
-    static __device__ __forceinline__ void store(unsigned char *buf, int site, double v, uint32_t seq)
-    {
-        st_raw((Raw16 *)buf + site, (unsigned long long)__double_as_longlong(v), seq);
-    }
-};
-
-template <>
-struct Packet<float> {
-    using Raw = unsigned long long;
-    static __device__ __forceinline__ Raw load(const unsigned char *buf, int site)
-    {
-        return ld_relaxed_u64((const unsigned long long *)buf + site);
-    }
-    static __device__ __forceinline__ bool ready(const Raw &r, uint32_t seq) { return (uint32_t)(r >> 32) == seq; }
-    static __device__ __forceinline__ float value(const Raw &r) { return __uint_as_float((uint32_t)r); }
-    static __device__ __forceinline__ void store(unsigned char *buf, int site, float v, uint32_t seq)
-    {
-        const unsigned long long w = ((unsigned long long)seq << 32) | __float_as_uint(v);
-        asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"((unsigned long long *)buf + site), "l"(w)
-                     : "memory");
-    }
-};
-
-// A bounded wait's clock: called once per failed poll; false when the budget
-// is spent or another block has recorded an error.
-struct SpinClock {
-    unsigned spins = 0;
-    uint64_t t0 = 0;
-    __device__ __forceinline__ bool tick(EngCtl *ctl)
-    {
-        if ((++spins & 63u) != 0) return true;
-        if (t0 == 0) t0 = global_ns();
-        if (ld_volatile_i32(&ctl->error) != 0) return false;
-        if ((long long)(global_ns() - t0) > ctl->timeout_ns) {
-            atomicCAS(&ctl->error, 0, -6);
-            return false;
-        }
-        return true;
-    }
-};
-
-// U packets of a thread (site < 0: none): all loads in flight at once, then
-// polled until each carries 'seq'.  False when the wait ran out.
-template <typename T, int U>
-__device__ __forceinline__ bool fetch(const unsigned char *buf, const int (&site)[U], uint32_t seq, T (&v)[U],
-                                      EngCtl *ctl)
-{
-    typename Packet<T>::Raw raw[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u)
-        if (site[u] >= 0) raw[u] = Packet<T>::load(buf, site[u]);
-    unsigned pend = 0;
-#pragma unroll
-    for (int u = 0; u < U; ++u)
-        if (site[u] >= 0) {
-            v[u] = Packet<T>::value(raw[u]);
-            if (!Packet<T>::ready(raw[u], seq)) pend |= 1u << u;
-        }
-    SpinClock clk;
-    while (pend) {
-        if (!clk.tick(ctl)) return false;
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-            if (pend & (1u << u)) {
-                const typename Packet<T>::Raw r = Packet<T>::load(buf, site[u]);
-                if (Packet<T>::ready(r, seq)) {
-                    v[u] = Packet<T>::value(r);
-                    pend &= ~(1u << u);
-                }
-            }
-    }
-    return true;
-}
-
-// All 32 lanes of a warp: the sum of n partial-sum packets once each carries
-// 'seq' (lane-strided sums in order, then a fixed tree; the same bits in every
-// lane of every block).  False in every lane when the wait ran out.
-__device__ __forceinline__ bool sum_slots(const Raw16 *slot, int n, uint32_t seq, EngCtl *ctl, double &sum)
-{
-    constexpr int U = 5;
-    const int lane = (int)(threadIdx.x & 31u);
-    double v = 0.0;
-    bool ok = true;
-    SpinClock clk;
-#pragma unroll 1
-    for (int j0 = 0; j0 < n && ok; j0 += 32 * U) {
-        Raw16 a[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            a[u].v = 0;
-            a[u].seq = seq;
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-            if (j0 + 32 * u + lane < n) a[u] = ld_raw(slot + j0 + 32 * u + lane);
-        while (true) {
-            bool ready = true;
-#pragma unroll
-            for (int u = 0; u < U; ++u) ready = ready && ((uint32_t)a[u].seq == seq);
-            if (ready) break;
-            if (!clk.tick(ctl)) {
-                ok = false;
-                break;
-            }
-#pragma unroll
-            for (int u = 0; u < U; ++u)
-                if ((uint32_t)a[u].seq != seq) a[u] = ld_raw(slot + j0 + 32 * u + lane);
-        }
-        const double a01 = __longlong_as_double((long long)a[0].v) + __longlong_as_double((long long)a[1].v);
-        const double a23 = __longlong_as_double((long long)a[2].v) + __longlong_as_double((long long)a[3].v);
-        v += (a01 + a23) + __longlong_as_double((long long)a[4].v);
-    }
-    ok = __all_sync(0xffffffffu, ok);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    sum = v;
-    return ok;
-}
-
-// Sum over a warp of non-negative values, in integers: each value's significand,
-// shifted to the largest exponent of the warp, in three 27-bit parts that the
-// integer warp reduction adds exactly (81 bits; what is shifted out is below
-// 2^-80 of the largest value).  The same result in every lane; NaN if a value
-// is not finite.  The shuffle tree of FP64 adds takes 5 x 16 cycles of the
-// SM's FP64 pipe per warp, 1.4k cycles for 16 warps; this takes none of it.
-struct SumParts {
-    int e;                  // biased FP64 exponent
-    unsigned long long m;   // significand, 53 bits
-};
-
-__device__ __forceinline__ SumParts sum_parts(double v)
-{
-    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-    SumParts p;
-    p.e = (int)((b >> 52) & 0x7ffu);
-    p.m = b & 0xfffffffffffffull;
-    if (p.e)
-        p.m |= 1ull << 52;
-    else
-        p.e = 1;
-    return p;
-}
-
-__device__ __forceinline__ SumParts sum_parts(float v)
-{
-    const unsigned b = __float_as_uint(v);
-    int e = (int)((b >> 23) & 0xffu);
-    unsigned m = b & 0x7fffffu;
-    if (e)
-        m |= 1u << 23;
-    else
-        e = 1;
-    SumParts p;
-    p.e = e == 255 ? 0x7ff : e + (1023 - 127);
-    p.m = (unsigned long long)m << 29;
-    return p;
-}
-
-template <typename T>
-__device__ __forceinline__ double warp_sum_nonneg(T v)
-{
-    const SumParts p = sum_parts(v);
-    const int emax = (int)__reduce_max_sync(0xffffffffu, (unsigned)p.e);
-    const int d = emax - p.e;
-    // m 2^28 >> d as 81 bits: parts of bits [54, 81), [27, 54), [0, 27).
-    unsigned a2 = 0, a1 = 0, a0 = 0;
-    if (d <= 80) {
-        const unsigned long long hi = d < 64 ? p.m >> d : 0ull;                       // bits from 28 up
-        const unsigned long long lo = d == 0 ? 0ull : d < 64 ? p.m << (64 - d) : d == 64 ? p.m : p.m >> (d - 64);
-        a2 = (unsigned)(hi >> 26);
-        a1 = (unsigned)(hi << 1) & 0x7ffffffu;
-        a1 |= (unsigned)(lo >> 63);
-        a0 = (unsigned)(lo >> 36) & 0x7ffffffu;
-    }
-    const unsigned long long s2 = __reduce_add_sync(0xffffffffu, a2);
-    const unsigned long long s1 = __reduce_add_sync(0xffffffffu, a1);
-    const unsigned long long s0 = __reduce_add_sync(0xffffffffu, a0);
-    if (emax == 0x7ff) return __longlong_as_double((long long)kSigNaN);
-    // S = s2 2^54 + s1 2^27 + s0 in units of 2^(emax - 1023 - 80): its upper 64
-    // bits (below them: a sticky bit) rounded to nearest even.
-    const unsigned long long l = s0 + ((s1 & 0x1fffffffffull) << 27);   // < 2^60
-    unsigned long long h = s2;                                          // units of 2^54
-    const unsigned long long c = l >> 54;
-    h += c;
-    const unsigned long long rest = l & 0x3fffffffffffffull;            // 54 bits
-    if (h == 0 && rest == 0) return 0.0;
-    // h has up to 33 bits: with rest 87.  Normalise so that the top bit is bit 63.
-    const int z = h ? __clzll((long long)h) : 0;
-    unsigned long long t;
-    int e;
-    if (h) {
-        t = (h << z) | (z ? ((rest << 10) >> (64 - z)) : 0ull);
-        const unsigned long long low = z ? (rest << 10) << z : (rest << 10);
-        t |= low != 0 ? 1ull : 0ull;
-        e = 63 - z + 54;
-    } else {
-        const int zr = __clzll((long long)rest);
-        t = rest << zr;
-        e = 63 - zr;
-    }
-    // t in [2^63, 2^64), value t 2^(e - 63) units.
-    unsigned long long m = t >> 11;
-    const unsigned long long frac = t & 0x7ffull;
-    m += (frac > 0x400ull || (frac == 0x400ull && (m & 1))) ? 1ull : 0ull;
-    e += emax - 80;                     // biased exponent of the result
-    if (e <= 0) return __longlong_as_double((long long)(m >> (e < -51 ? 53 : 1 - e)));
-    if (e >= 0x7ff) return __longlong_as_double((long long)kSigNaN);
-    return __longlong_as_double((long long)(((unsigned long long)(e - 1) << 52) + m));
-}
 
 // ---------------------------------------------------------------------------
 // The kernel.  D: lattice dimension; T: type of the CG steps (float: mixed
@@ -303,8 +56,10 @@ __global__ void __launch_bounds__(kOcMaxThreads, 1) k_onchip(const OcLaunch L)
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ EngSystem s_sys;
     __shared__ EngState s_st;
-    __shared__ double s_red[kOcMaxThreads / 32];
-    __shared__ double s_scal;       // beta or alpha of the phase about to run
+    __shared__ ISum s_red[kOcMaxThreads / 32];
+    __shared__ double s_redd[kOcMaxThreads / 32];    // signed sums
+    __shared__ T s_scal;            // beta or alpha of the phase about to run
+    __shared__ int s_restart;       // beta = 0: p starts anew
     __shared__ double s_tolbb, s_dmax;   // tol^2 |b|^2 and delta^2 maxr2 of the fast decision
     __shared__ int s_hand;          // a mixed system leaves for FP64 steps in the grid engine
 
@@ -379,25 +134,35 @@ __global__ void __launch_bounds__(kOcMaxThreads, 1) k_onchip(const OcLaunch L)
     int par = 0;        // parity of the partial-sum packets
     const bool drop = L.drop != 0 && L.drop - 1 == tile && sid == 0;
     const int nwarp = nthr >> 5;
-    const int wtop = nwarp <= 1 ? 0 : nwarp <= 2 ? 1 : nwarp <= 4 ? 2 : nwarp <= 8 ? 4 : 8;
 
-    // Publishes the block's sum under the current phase number, from each
-    // warp's sum (every thread calls it; its barrier follows all of the block's
-    // writes of the phase).
-    auto publish = [&](double wsum) {
-        if ((tid & 31) == 0) s_red[tid >> 5] = wsum;
+    // Publishes the block's sum of v under the current phase number (every thread
+    // calls it; its barrier follows all of the block's writes of the phase).
+    auto publish_value = [&](double v) {
+        if (tid < kOcReplicas && !drop)
+            st_raw(slots + (size_t)(2 * tid + par) * kOcMaxTiles + tile,
+                   (unsigned long long)__double_as_longlong(v), ph);
+    };
+    auto publish = [&](auto v) {
+        const ISum a = warp_isum(v);
+        if ((tid & 31) == 0) s_red[tid >> 5] = a;
         __syncthreads();
         if (tid < 32) {
-            double w = tid < nwarp ? s_red[tid] : 0.0;
-            for (int o = wtop; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
-            if (tid < kOcReplicas && !drop)
-                st_raw(slots + (size_t)(2 * tid + par) * kOcMaxTiles + tile,
-                       (unsigned long long)__double_as_longlong(__shfl_sync((1u << kOcReplicas) - 1u, w, 0)), ph);
+            ISum b = {0ull, 1};
+            if (tid < nwarp) b = s_red[tid];
+            publish_value(isum_value(warp_isum_parts(b)));
         }
     };
-    // Warp 0: waits for the sum published last.
-    auto wait_sum = [&](double &sum) -> bool {
-        return sum_slots(my_slots + par * kOcMaxTiles, tiles, ph, ctl, sum);
+    // The same for a sum of either sign.
+    auto publish_signed = [&](double v) {
+        v = warp_sum(v);
+        if ((tid & 31) == 0) s_redd[tid >> 5] = v;
+        __syncthreads();
+        if (tid < 32) {
+            double w = tid < nwarp ? s_redd[tid] : 0.0;
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+            publish_value(__shfl_sync(0xffffffffu, w, 0));
+        }
     };
     // A barrier over the system's tiles that also orders plain global accesses.
     // Returns true when a wait ran out.
@@ -411,7 +176,7 @@ __global__ void __launch_bounds__(kOcMaxThreads, 1) k_onchip(const OcLaunch L)
             if (tid < kOcReplicas && !drop) st_raw(slots + (size_t)(2 * tid + par) * kOcMaxTiles + tile, 0ull, ph);
             __syncwarp();
             double dummy;
-            bad = !wait_sum(dummy);
+            bad = !sum_slots<true>(my_slots + par * kOcMaxTiles, tiles, ph, ctl, dummy);
             __threadfence();
         }
         return __syncthreads_or(bad ? 1 : 0) != 0;
@@ -477,46 +242,44 @@ __global__ void __launch_bounds__(kOcMaxThreads, 1) k_onchip(const OcLaunch L)
 
     bool bad = false;
     bool stageB = false;    // the next exchange brings t (and |t|^2), else M's input (and |r|^2)
-    int pm = s_st.mode;     // mode of the phases run last
+    int pm = MODE_NEW;      // mode of the phases run last
+    int pj = 0;             // preconditioner sub-step (s_st.pre_j may already be the next)
     long long iters = 0;
     __syncthreads();
     for (;;) {
         // ---- exchange: warp 0 waits for the sum of the last phase and turns it
         // into the next scalar (and mode), the other warps fetch the halo ----
         const int cheb2 = CHEB ? 2 * Y.cheb_n : 0;
+        bool again = false;     // warp 0: another CG step, its state noted after the barrier
+        double sum = 0.0;
         if (tid < 32) {
             // Between the preconditioner's sub-steps there is no sum.
             const bool inner = CHEB && pm == MODE_PRE && (stageB || s_st.pre_j + 1 < cheb2);
             __syncwarp();
             if (!inner && pm != MODE_NEW) {
-                const double ra = s_st.rr_alpha;
-                double inv = 0.0, sum;
-                if (!stageB) inv = 1.0 / ra;        // off the critical path: used when the sum arrives
-                if (!wait_sum(sum)) {
+                const double ra = s_st.rr_alpha, inv = stageB ? 0.0 : reciprocal(ra);
+                const double tolbb = s_tolbb, dmax = MIXED ? s_dmax : 0.0;
+                const bool last = s_st.cg_steps + 1 >= Y.maxit || (MIXED && s_st.since_ru + 1 >= Y.stall_window);
+                const bool ok = CHEB && pm == MODE_PRE
+                                    ? sum_slots<false>(my_slots + par * kOcMaxTiles, tiles, ph, ctl, sum)
+                                    : sum_slots<true>(my_slots + par * kOcMaxTiles, tiles, ph, ctl, sum);
+                if (!ok) {
                     bad = true;
                 } else if (stageB) {
-                    if (tid == 0) s_scal = ra / sum;
+                    const T a = quotient<T>(ra, sum);
+                    if (tid == 0) s_scal = a;
                 } else {
-                    const int steps = s_st.cg_steps + 1, since = s_st.since_ru + 1;
-                    const bool stop = !(sum > s_tolbb) || (MIXED && sum < s_dmax) || !isfinite(sum) ||
-                                      (MIXED && since >= Y.stall_window) || steps >= Y.maxit;
-                    if (!CHEB && pm == MODE_CG && !stop) {
-                        // The common case of decide(): another CG step, beta = sum / ra
-                        // (the quotient by 1 / ra with one residual correction).
+                    again = !CHEB && pm == MODE_CG && !last && finite_bits(sum) && greater_nonneg(sum, tolbb) &&
+                            !(MIXED && greater_nonneg(dmax, sum));
+                    if (again) {
+                        // The common case of decide(): beta = sum / ra, the quotient by
+                        // 1 / ra with (FP64) one residual correction.
+                        double beta = sum * inv;
+                        if (!MIXED) beta = fma(fma(-beta, ra, sum), inv, beta);
                         if (tid == 0) {
-                            double beta = sum * inv;
-                            beta = fma(fma(-beta, ra, sum), inv, beta);
-                            s_scal = beta;
+                            s_scal = (T)beta;
+                            s_restart = 0;
                             s_st.beta = beta;
-                            s_st.cg_steps = steps;
-                            s_st.since_ru = since;
-                            if (!MIXED) s_st.fp64_steps += 1;
-                            s_st.rr_last = sum;
-                            s_st.rr_alpha = sum;
-                            if (MIXED && sum > s_st.maxr2) {
-                                s_st.maxr2 = sum;
-                                s_dmax = Y.delta2 * sum;
-                            }
                         }
                     } else if (tid == 0) {
                         const EngState S = decide(Y, s_st, sum);
@@ -524,16 +287,11 @@ __global__ void __launch_bounds__(kOcMaxThreads, 1) k_onchip(const OcLaunch L)
                             // FP64 steps of a mixed system: the grid engine goes on from
                             // this reliable update (its state and |r|^2, x, r in memory).
                             s_hand = 1;
-                            if (tile == 0) {
-                                for (int j = 0; j < Y.ntiles; ++j)
-                                    L.sig[(size_t)5 * L.sig_stride + Y.part0 + j] =
-                                        (unsigned long long)__double_as_longlong(j == 0 ? sum : 0.0);
-                                L.state[0][sid] = s_st;
-                                L.state[1][sid] = s_st;
-                            }
+                            if (tile == 0) hand_over(L, Y, sid, s_st, sum);
                         } else {
                             s_st = S;
-                            s_scal = S.beta;
+                            s_scal = (T)S.beta;
+                            s_restart = S.beta == 0.0;
                             s_tolbb = Y.tol2 * S.bb;
                             s_dmax = Y.delta2 * S.maxr2;
                         }
@@ -553,13 +311,24 @@ __global__ void __launch_bounds__(kOcMaxThreads, 1) k_onchip(const OcLaunch L)
         }
         if (iters >= L.max_iters) bad = true;
         if (__syncthreads_or(bad ? 1 : 0)) break;
+        if (again && tid == 0) {
+            s_st.cg_steps += 1;
+            s_st.since_ru += 1;
+            if (!MIXED) s_st.fp64_steps += 1;
+            s_st.rr_last = sum;
+            s_st.rr_alpha = sum;
+            if (MIXED && sum > s_st.maxr2) {
+                s_st.maxr2 = sum;
+                s_dmax = Y.delta2 * sum;
+            }
+        }
 
         if (stageB) {
             stageB = false;
             ++ph;
             if (CHEB && pm == MODE_PRE) {
                 // Factor update of a preconditioner sub-step.
-                const int j = s_st.pre_j, k = j >> 1;
+                const int j = pj, k = j >> 1;
                 const bool last = j == cheb2 - 1;
                 const T invlam = (T)__ldg(Y.cheb), a = (T)__ldg(Y.cheb + 2 + 3 * k);
                 const T b2 = (T)__ldg(Y.cheb + 3 + 3 * k), invq = (T)__ldg(Y.cheb + 4 + 3 * k);
@@ -580,18 +349,18 @@ __global__ void __launch_bounds__(kOcMaxThreads, 1) k_onchip(const OcLaunch L)
                             if (last) acc = fma((double)Rb[s], (double)w, acc);
                         }
                         Sb[RS + e] = w;
-                        if (tl == st - 1 || r < P || r >= row - P) PK::store(pktA, gbase + s + tl * gstep, w, ph);
+                        if (tl == st - 1 || r < P || r >= row - P) PK::store((typename PK::Raw *)pktA + gbase + s + tl * gstep, w, ph);
                     }
                 });
                 if (last) {
                     par ^= 1;
-                    publish(warp_sum(acc));
+                    publish_signed(acc);
                 }
                 continue;
             }
             // ---- r -= alpha M^T t, |r|^2; then x += alpha p while the sum travels ----
-            const T alpha = (T)s_scal;
-            T sum = T(0);
+            const T alpha = s_scal;
+            T acc = T(0);
             par ^= 1;
             sites([&](int s0, auto un) {
 #pragma unroll
@@ -602,11 +371,11 @@ __global__ void __launch_bounds__(kOcMaxThreads, 1) k_onchip(const OcLaunch L)
                     const T r = fma(-alpha, y, CHEB ? Rb[s] : Sb[RS + e]);
                     Sb[RS + e] = r;
                     if (CHEB) Rb[s] = r;
-                    sum = fma(r, r, sum);
-                    if (tl == st - 1 || ro < P || ro >= row - P) PK::store(pktA, gbase + s + tl * gstep, r, ph);
+                    acc = fma(r, r, acc);
+                    if (tl == st - 1 || ro < P || ro >= row - P) PK::store((typename PK::Raw *)pktA + gbase + s + tl * gstep, r, ph);
                 }
             });
-            publish(warp_sum_nonneg(sum));
+            publish(acc);
             sites([&](int s0, auto un) {
 #pragma unroll
                 for (int u = 0; u < un.value; ++u) {
@@ -643,7 +412,7 @@ __global__ void __launch_bounds__(kOcMaxThreads, 1) k_onchip(const OcLaunch L)
                 acc = fma(b, b, acc);
                 Sb[RS + e] = (T)b;
                 if (CHEB) Rb[s] = (T)b;
-                if (tl == st - 1 || r < P || r >= row - P) PK::store(pktA, g, (T)b, ph);
+                if (tl == st - 1 || r < P || r >= row - P) PK::store((typename PK::Raw *)pktA + g, (T)b, ph);
                 const double x = zero ? 0.0 : Y.x[g];
                 if (MIXED) {
                     if (zero) Y.x[g] = 0.0;
@@ -657,7 +426,7 @@ __global__ void __launch_bounds__(kOcMaxThreads, 1) k_onchip(const OcLaunch L)
                     Y.x[g] = 0.0;
                 }
             }
-            publish(warp_sum(acc));
+            publish(acc);
             pm = mode;
             continue;
         }
@@ -696,9 +465,9 @@ __global__ void __launch_bounds__(kOcMaxThreads, 1) k_onchip(const OcLaunch L)
                 Sb[RS + s + P + 2 * P * tl] = (T)res;
                 if (CHEB) Rb[s] = (T)res;
                 if (MIXED) Y.r[g] = res;
-                if (tl == st - 1 || r < P || r >= row - P) PK::store(pktA, g, (T)res, ph);
+                if (tl == st - 1 || r < P || r >= row - P) PK::store((typename PK::Raw *)pktA + g, (T)res, ph);
             }
-            publish(warp_sum(acc));
+            publish(acc);
             pm = mode;
             continue;
         }
@@ -708,8 +477,8 @@ __global__ void __launch_bounds__(kOcMaxThreads, 1) k_onchip(const OcLaunch L)
         // its halo ----
         const bool cg = !CHEB || mode == MODE_CG;
         if (cg) {
-            const bool restart = s_st.beta == 0.0;
-            const T beta = (T)s_scal;
+            const bool restart = s_restart != 0;
+            const T beta = s_scal;
             const int E = (st + 1) * RS;
             int j = tid;
 #pragma unroll 1
@@ -736,14 +505,15 @@ __global__ void __launch_bounds__(kOcMaxThreads, 1) k_onchip(const OcLaunch L)
                 const T y = fma(Lb[s], v[e], fma(-h, hop(v + RS, e, s), v[RS + e]));
                 Tb[e] = y;
                 if (cg) acc = fma(y, y, acc);
-                if (tl == 0 || r < P || r >= row - P) PK::store(pktB, gbase + s + tl * gstep, y, ph);
+                if (tl == 0 || r < P || r >= row - P) PK::store((typename PK::Raw *)pktB + gbase + s + tl * gstep, y, ph);
             }
         });
         if (cg) {
             par ^= 1;
-            publish(warp_sum_nonneg(acc));
+            publish(acc);
         }
         stageB = true;
+        pj = pm == MODE_PRE ? pj + 1 : 0;
         pm = mode;
     }
 
@@ -786,7 +556,56 @@ size_t oc_smem(int d, long long P, int so, int st, bool mixed, bool cheb, bool x
 
 }  // namespace
 
-OcPlan oc_plan(int d, int nx, int ntau, int nsys, bool mixed, bool cheb, int nsm, size_t smem_sm, size_t smem_blk)
+// Column form: a tile's row of so P sites, one per thread, st slices each, with
+// one halo column per edge thread, or two when tiles have one o position (d = 3).
+static bool cols_candidate(int d, long long P, int nx, int go, int so, int st, bool mixed, bool cheb, int *K,
+                           int *sides, int *threads)
+{
+    const long long row = P * so;
+    if (row > kColMaxRow || st > (cheb ? 4 : 8)) return false;
+    *sides = nx / go >= 2 ? 1 : 2;
+    if (*sides == 2 && (d == 1 || so != 1)) return false;
+    *K = st <= 2 ? 2 : st <= 4 ? 4 : 8;
+    *threads = (int)((row + 31) / 32 * 32) + 32;
+    return *threads <= col_max_threads(mixed ? 4 : 8, *K);
+}
+
+static const void *plan_kernel(const OcPlan &P, int d)
+{
+    return P.cols ? oc_cols_kernel(d, P.mixed != 0, P.cheb != 0, P.cols, P.sides) : oc_kernel(d, P.mixed != 0, P.cheb != 0);
+}
+
+// Registers per thread of a layout's kernel, asked once per process.
+static int kernel_regs(const OcPlan &P, int d)
+{
+    static std::atomic<int> known[2 * 2 * 2 * 3 * 9];
+    std::atomic<int> &k =
+        known[(((d == 3) * 2 + (P.mixed != 0)) * 2 + (P.cheb != 0)) * 27 + P.sides * 9 + P.cols];
+    int r = k.load(std::memory_order_relaxed);
+    if (r == 0) {
+        cudaFuncAttributes a;
+        if (cudaFuncGetAttributes(&a, plan_kernel(P, d)) != cudaSuccess) {
+            cudaGetLastError();
+            return 0;
+        }
+        r = a.numRegs;
+        k.store(r, std::memory_order_relaxed);
+    }
+    return r;
+}
+
+int oc_max_blocks(const OcPlan &P, int d)
+{
+    const void *fn = plan_kernel(P, d);
+    int per = 0;
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kOcMaxSmem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, P.threads, P.smem) != cudaSuccess)
+        return 0;
+    return per;
+}
+
+OcPlan oc_plan(int d, int nx, int ntau, int nsys, bool mixed, bool cheb, int nsm, size_t smem_sm, size_t smem_blk,
+               int forms)
 {
     OcPlan best = {};
     const long long P = d == 3 ? (long long)nx * nx : 1;
@@ -803,51 +622,67 @@ OcPlan oc_plan(int d, int nx, int ntau, int nsys, bool mixed, bool cheb, int nsm
             for (int st = 1, gt; st <= ntau; st = gt == 1 ? ntau + 1 : (ntau + gt - 2) / (gt - 1)) {
                 gt = (ntau + st - 1) / st;
                 if ((long long)go * gt > G) continue;
-                for (int xg = 0; xg < 2; ++xg) {
-                    const size_t sm = oc_smem(d, P, so, st, mixed, cheb, xg != 0);
+                const long long C = P * so * st, H = P * (2 * st + so);
+                for (int form = forms == 2 ? 1 : 0; form < (forms == 3 ? 1 : 3); ++form) {
+                    // form 0: columns; 1, 2: tile form with x in shared or global memory
+                    int K = 0, sides = 1, thr = 0;
+                    size_t sm;
+                    // Clocks of one iteration on an SM holding m tiles, from times measured over so,
+                    // st and m on the lattices of the size range (within about 10% of them).
+                    double cost;
+                    if (form == 0) {
+                        if (!cols_candidate(d, P, nx, go, so, st, mixed, cheb, &K, &sides, &thr)) continue;
+                        sm = oc_cols_smem(d, mixed, cheb, K, thr);
+                        const double warps = (thr - 32) / 32;
+                        cost = 7000.0 + 20.0 * go * gt + (sides == 2 ? 2500.0 : 0.0) + (cheb && K > 2 ? 1500.0 : 0.0) +
+                               (!mixed && K == 8 ? 2500.0 : 0.0) +
+                               (mixed ? 300.0 : 500.0) * st +
+                               m * (warps * st * (mixed ? 22.0 * d : 16.0 * (d == 1 ? 12 : 20)) + 0.5 * H);
+                    } else {
+                        sm = oc_smem(d, P, so, st, mixed, cheb, form == 2);
+                        thr = (int)((C + 31) / 32 * 32);
+                        // More than 8 warps only lengthen the block's barriers and sums while
+                        // a thread has few sites.
+                        if (thr > 256 && C <= 2048) thr = 256;
+                        if (thr > max_threads) thr = max_threads;
+                        if (thr < 64) thr = 64;
+                        const double site = mixed ? 2.6 : d == 1 ? 6.5 : 13.0;
+                        cost = 9500.0 + 20.0 * go * gt + m * (C * (site + (form == 2 ? 0.5 : 0.0)) + 0.7 * H);
+                    }
                     if (sm > kOcMaxSmem || sm + kStatic > smem_blk || (sm + kStatic) * m > smem_sm) continue;
-                    const long long C = P * so * st, H = P * (2 * st + so);
-                    // Clocks of one phase on an SM holding m tiles.
-                    const double site = mixed ? 0.8 : 3.0;
-                    const double cost = m * (C * (site + (xg ? 0.3 : 0.0)) + H * 1.0) + 10.0 * go * gt;
                     if (best.ok && cost >= best_cost) continue;
+                    OcPlan p = {};
+                    p.ok = 1;
+                    p.go = go;
+                    p.gt = gt;
+                    p.so = so;
+                    p.st = st;
+                    p.x_global = form == 2;
+                    p.mixed = mixed;
+                    p.cheb = cheb;
+                    p.cols = K;
+                    p.sides = sides;
+                    p.smem = sm;
+                    p.threads = thr;
+                    // Co-resident, as its blocks wait on one another: by registers (a
+                    // warp's are one of the 4 partitions', 16384 each) and shared memory.
+                    const int regs = (kernel_regs(p, d) + 7) / 8 * 8;
+                    const int parts = (thr / 32 + 3) / 4;    // warps of a block per partition
+                    if (regs <= 0 || 16384 / (regs * 32) / parts < m) continue;
                     best_cost = cost;
-                    best.ok = 1;
-                    best.go = go;
-                    best.gt = gt;
-                    best.so = so;
-                    best.st = st;
-                    best.x_global = xg;
-                    best.mixed = mixed;
-                    best.cheb = cheb;
-                    best.smem = sm;
-                    // More than 8 warps only lengthen the block's barriers and sums while
-                    // a thread has few sites.
-                    int thr = (int)((C + 31) / 32 * 32);
-                    if (thr > 256 && C <= 2048) thr = 256;
-                    if (thr > max_threads) thr = max_threads;
-                    if (thr < 64) thr = 64;
-                    best.threads = thr;
+                    best = p;
                 }
             }
         }
     }
+    // The occupancy calculation has the last word.
+    if (best.ok && oc_max_blocks(best, d) * nsm < best.go * best.gt * nsys) best.ok = 0;
     return best;
-}
-
-int oc_max_blocks(const OcPlan &P, int d)
-{
-    const void *fn = oc_kernel(d, P.mixed != 0, P.cheb != 0);
-    int per = 0;
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kOcMaxSmem) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, P.threads, P.smem) != cudaSuccess)
-        return 0;
-    return per;
 }
 
 cudaError_t oc_launch(const OcLaunch &L, const OcPlan &P, int d, cudaStream_t st)
 {
-    const void *fn = oc_kernel(d, P.mixed != 0, P.cheb != 0);
+    const void *fn = plan_kernel(P, d);
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kOcMaxSmem);
     if (e != cudaSuccess) return e;
     OcLaunch arg = L;
