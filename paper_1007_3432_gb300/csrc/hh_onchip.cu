@@ -29,9 +29,9 @@
 // warps (FP64 from about 800 sites per SM: the FP64 pipe, 16 clocks per warp
 // instruction).  Measured against the grid engine, us per iteration: d = 1
 // 1024 x 128 FP64, 2 right-hand sides, 10.5 (15.4), a degree-8 preconditioned
-// step on 256 x 256 91 (199); d = 3 16^3 x 64 mixed, one, 8.2 (15.1), two, 8.5
-// (16.5), 20^3 x 96 mixed, one, 11.3 (18.2).  It was faster wherever the vectors
-// fit (20^3 x 64 mixed, two: 15.1 against 19.4).  Tiles whose column fits a
+// step on 256 x 256 89 (199); d = 3 16^3 x 64 mixed, one, 6.9 (15.1), two, 7.7
+// (16.5), 20^3 x 96 mixed, one, 10.5 (18.2).  It was faster wherever the vectors
+// fit (20^3 x 64 mixed, two: 13.7 against 19.4).  Tiles whose column fits a
 // thread's registers run in hh_onchip_cols.cu.
 //
 // Every wait is bounded (EngCtl::timeout_ns); on expiry the block records
@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(kOcMaxThreads, 1) k_onchip(const OcLaunch L)
     T *const Rb = q;                    // preconditioner: r and z, compact
     T *const Zb = q + (CHEB ? maxC : 0);
     q += CHEB ? 2 * maxC : 0;
-    unsigned char *const fl = (unsigned char *)q;    // d = 3: x-y edges of each compact site
+    unsigned char *const fl = (unsigned char *)q;    // d = 3: x-y edges of each spatial site of the row
     T *const Xg = MIXED ? (T *)Y.x32 : (T *)Y.x;
 
     unsigned char *const pktA = L.pkt + (size_t)sid * 2 * L.N * sizeof(typename PK::Raw);
@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(kOcMaxThreads, 1) k_onchip(const OcLaunch L)
 
     const T h = (T)Y.h;
     if (D == 3)
-        for (int s = tid; s < C; s += nthr) {
+        for (int s = tid; s < row; s += nthr) {
             const int pos = s - (int)fd_div((uint32_t)s, f_P) * P;
             const int y = pos / nx, x = pos - y * nx;
             fl[s] = (unsigned char)((x == 0) | (x == nx - 1) << 1 | (y == 0) << 2 | (y == nx - 1) << 3);
@@ -183,6 +183,7 @@ __global__ void __launch_bounds__(kOcMaxThreads, 1) k_onchip(const OcLaunch L)
     };
 
     const int H2 = 2 * st * P, HA = H2 + row;
+    const FastDiv f_2P = make_fastdiv((uint32_t)(2 * P));
     // Halo threads: all but warp 0 (which waits for the sums) when there are others.
     const int hb = nwarp > 1 ? tid - 32 : tid, hn = nwarp > 1 ? nthr - 32 : nthr;
     // The halo of the packets in buf: o columns of the tile's rows into side (extended),
@@ -190,7 +191,38 @@ __global__ void __launch_bounds__(kOcMaxThreads, 1) k_onchip(const OcLaunch L)
     auto fetch_halo = [&](const unsigned char *buf, T *side, T *rdst, int grow) -> bool {
         constexpr int U = 4;
         bool ok = true;
-        if (hb >= 0)
+        if (hb < 0) return ok;
+        if constexpr (MIXED) {
+            // Up to U slices of one column site at a time, then the row.
+#pragma unroll 1
+            for (int i = hb; i < 2 * P * ((st + U - 1) / U) && ok; i += hn) {
+                const int q4 = (int)fd_div((uint32_t)i, f_2P), cs = i - q4 * 2 * P, k0 = q4 * U;
+                int g = (t0 + k0) * V + (cs < P ? oL + cs : oR + cs - P);
+                T *dst = side + k0 * RS + (cs < P ? cs : RS - 2 * P + cs);
+                HH_CHECK(g, 0, L.N, BC_NEIGHBOUR);
+                int hg[U];
+                T v[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) hg[u] = k0 + u < st ? g + u * V : -1;
+                ok = fetch<T, U>(buf, hg, ph, v, ctl);
+#pragma unroll
+                for (int u = 0; u < U; ++u, dst += RS)
+                    if (hg[u] >= 0) *dst = v[u];
+            }
+#pragma unroll 1
+            for (int j = hb; j < row && ok; j += U * hn) {
+                int g = grow + j;
+                HH_CHECK(g, 0, L.N, BC_NEIGHBOUR);
+                int hg[U];
+                T v[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) hg[u] = j + u * hn < row ? g + u * hn : -1;
+                ok = fetch<T, U>(buf, hg, ph, v, ctl);
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (hg[u] >= 0) rdst[j + u * hn] = v[u];
+            }
+        } else {
 #pragma unroll 1
             for (int j0 = hb; j0 < HA && ok; j0 += U * hn) {
                 int hg[U];
@@ -218,13 +250,14 @@ __global__ void __launch_bounds__(kOcMaxThreads, 1) k_onchip(const OcLaunch L)
                 for (int u = 0; u < U; ++u)
                     if (hg[u] >= 0) *dst[u] = v[u];
             }
+        }
         return ok;
     };
 
     // Hopping sum around extended index e of array v.
-    auto hop = [&](const T *v, int e, int s) -> T {
+    auto hop = [&](const T *v, int e, int c) -> T {
         if (D == 1) return v[e + 1] + v[e - 1];
-        const unsigned f = fl[s];
+        const unsigned f = fl[c];
         const T xr = v[f & 2u ? e - (nx - 1) : e + 1], xl = v[f & 1u ? e + (nx - 1) : e - 1];
         const T yp = v[f & 8u ? e - (nx - 1) * nx : e + nx], ym = v[f & 4u ? e + (nx - 1) * nx : e - nx];
         return (xr + xl) + ((yp + ym) + (v[e + P] + v[e - P]));
@@ -238,6 +271,45 @@ __global__ void __launch_bounds__(kOcMaxThreads, 1) k_onchip(const OcLaunch L)
         for (; s + (UN - 1) * nthr < C; s += UN * nthr) f(s, std::integral_constant<int, UN>{});
 #pragma unroll 1
         for (; s < C; s += nthr) f(s, std::integral_constant<int, 1>{});
+    };
+
+    // ---- FP32: work items of up to kSlices consecutive slices of one spatial site, so
+    // that the index arithmetic is done once for them and the time neighbours of all but
+    // the ends are in registers (16^3 x 64, one right-hand side: 8.2 -> 6.8 us per
+    // iteration).  FP64 keeps the strided sites above, whose chains overlap better
+    // (256 x 256 preconditioned: 91 us per step against 109) ----
+    constexpr int kSlices = 4;
+    const int nq = (st + kSlices - 1) / kSlices, items = row * nq;
+    struct Item {
+        int c, k0, n;           // row site, first slice, slices
+        int e;                  // extended index (rows from 0) of slice k0
+        int xr, xl, yp, ym;     // spatial neighbours from e
+        bool edge;              // an o edge of the tile: its halo sites are read elsewhere
+    };
+    auto item = [&](int i) -> Item {
+        Item w;
+        const int q4 = (int)fd_div((uint32_t)i, f_row);
+        w.c = i - q4 * row;
+        w.k0 = q4 * kSlices;
+        w.n = st - w.k0 < kSlices ? st - w.k0 : kSlices;
+        w.e = w.k0 * RS + P + w.c;
+        w.edge = w.c < P || w.c >= row - P;
+        w.xr = 1;
+        w.xl = -1;
+        w.yp = w.ym = 0;
+        if (D == 3) {
+            const unsigned f = fl[w.c];
+            w.xr = f & 2u ? -(nx - 1) : 1;
+            w.xl = f & 1u ? nx - 1 : -1;
+            w.yp = f & 8u ? -(nx - 1) * nx : nx;
+            w.ym = f & 4u ? (nx - 1) * nx : -nx;
+        }
+        return w;
+    };
+    // Hopping sum around v (the item's site of one slice).
+    auto item_hop = [&](const T *v, const Item &w) -> T {
+        if (D == 1) return v[1] + v[-1];
+        return (v[w.xr] + v[w.xl]) + ((v[w.yp] + v[w.ym]) + (v[P] + v[-P]));
     };
 
     bool bad = false;
@@ -339,7 +411,7 @@ __global__ void __launch_bounds__(kOcMaxThreads, 1) k_onchip(const OcLaunch L)
                     for (int u = 0; u < un.value; ++u) {
                         const int s = s0 + u * nthr;
                         const int tl = (int)fd_div((uint32_t)s, f_row), e = s + P + 2 * P * tl, r = s - tl * row;
-                        const T y = fma(Lb[s + row], Tb[e + RS], fma(-h, hop(Tb, e, s), Tb[e])), v = Sb[RS + e];
+                        const T y = fma(Lb[s + row], Tb[e + RS], fma(-h, hop(Tb, e, r), Tb[e])), v = Sb[RS + e];
                         T w;
                         if ((j & 1) == 0) {
                             Zb[s] = v;
@@ -362,33 +434,77 @@ __global__ void __launch_bounds__(kOcMaxThreads, 1) k_onchip(const OcLaunch L)
             const T alpha = s_scal;
             T acc = T(0);
             par ^= 1;
-            sites([&](int s0, auto un) {
+            if constexpr (MIXED) {
+#pragma unroll 1
+                for (int i = tid; i < items; i += nthr) {
+                    const Item w = item(i);
+                    const T *tb = Tb + w.e;
+                    T *sb = Sb + RS + w.e;
+                    const T *lb = Lb + row + w.k0 * row + w.c;
+                    typename PK::Raw *pa = (typename PK::Raw *)pktA + gbase + w.c + w.k0 * V;
+                    T here = tb[0];
 #pragma unroll
-                for (int u = 0; u < un.value; ++u) {
-                    const int s = s0 + u * nthr;
-                    const int tl = (int)fd_div((uint32_t)s, f_row), e = s + P + 2 * P * tl, ro = s - tl * row;
-                    const T y = fma(Lb[s + row], Tb[e + RS], fma(-h, hop(Tb, e, s), Tb[e]));
-                    const T r = fma(-alpha, y, CHEB ? Rb[s] : Sb[RS + e]);
-                    Sb[RS + e] = r;
-                    if (CHEB) Rb[s] = r;
-                    acc = fma(r, r, acc);
-                    if (tl == st - 1 || ro < P || ro >= row - P) PK::store((typename PK::Raw *)pktA + gbase + s + tl * gstep, r, ph);
-                }
-            });
-            publish(acc);
-            sites([&](int s0, auto un) {
-#pragma unroll
-                for (int u = 0; u < un.value; ++u) {
-                    const int s = s0 + u * nthr;
-                    const int tl = (int)fd_div((uint32_t)s, f_row), e = s + P + 2 * P * tl;
-                    if (L.x_global) {
-                        T *const xp = Xg + gbase + s + tl * gstep;
-                        *xp = fma(alpha, Pb[RS + e], *xp);
-                    } else {
-                        Xb[s] = fma(alpha, Pb[RS + e], Xb[s]);
+                    for (int u = 0; u < kSlices; ++u) {
+                        if (u >= w.n) break;
+                        const T next = tb[RS];
+                        const T y = fma(*lb, next, fma(-h, item_hop(tb, w), here));
+                        const T r = fma(-alpha, y, *sb);
+                        *sb = r;
+                        acc = fma(r, r, acc);
+                        if (w.edge || w.k0 + u == st - 1) PK::store(pa, r, ph);
+                        here = next;
+                        tb += RS;
+                        sb += RS;
+                        lb += row;
+                        pa += V;
                     }
                 }
-            });
+            } else {
+                sites([&](int s0, auto un) {
+#pragma unroll
+                    for (int u = 0; u < un.value; ++u) {
+                        const int s = s0 + u * nthr;
+                        const int tl = (int)fd_div((uint32_t)s, f_row), e = s + P + 2 * P * tl, ro = s - tl * row;
+                        const T y = fma(Lb[s + row], Tb[e + RS], fma(-h, hop(Tb, e, ro), Tb[e]));
+                        const T r = fma(-alpha, y, CHEB ? Rb[s] : Sb[RS + e]);
+                        Sb[RS + e] = r;
+                        if (CHEB) Rb[s] = r;
+                        acc = fma(r, r, acc);
+                        if (tl == st - 1 || ro < P || ro >= row - P) PK::store((typename PK::Raw *)pktA + gbase + s + tl * gstep, r, ph);
+                    }
+                });
+            }
+            publish(acc);
+            if constexpr (MIXED) {
+#pragma unroll 1
+                for (int i = tid; i < items; i += nthr) {
+                    const int q4 = (int)fd_div((uint32_t)i, f_row), c = i - q4 * row, k0 = q4 * kSlices;
+                    const T *pb = Pb + RS + k0 * RS + P + c;
+                    const int step = L.x_global ? V : row;
+                    T *xp = L.x_global ? Xg + gbase + c + k0 * V : Xb + k0 * row + c;
+#pragma unroll
+                    for (int u = 0; u < kSlices; ++u) {
+                        if (k0 + u >= st) break;
+                        *xp = fma(alpha, *pb, *xp);
+                        pb += RS;
+                        xp += step;
+                    }
+                }
+            } else {
+                sites([&](int s0, auto un) {
+#pragma unroll
+                    for (int u = 0; u < un.value; ++u) {
+                        const int s = s0 + u * nthr;
+                        const int tl = (int)fd_div((uint32_t)s, f_row), e = s + P + 2 * P * tl;
+                        if (L.x_global) {
+                            T *const xp = Xg + gbase + s + tl * gstep;
+                            *xp = fma(alpha, Pb[RS + e], *xp);
+                        } else {
+                            Xb[s] = fma(alpha, Pb[RS + e], Xb[s]);
+                        }
+                    }
+                });
+            }
             continue;
         }
 
@@ -496,18 +612,44 @@ __global__ void __launch_bounds__(kOcMaxThreads, 1) k_onchip(const OcLaunch L)
         const T *const v = cg ? Pb : Sb;
         T acc = T(0);
         ++ph;
-        sites([&](int s0, auto un) {
+        if constexpr (MIXED) {
+#pragma unroll 1
+            for (int i = tid; i < items; i += nthr) {
+                const Item w = item(i);
+                const T *vb = v + RS + w.e;
+                T *tb = Tb + w.e;
+                const T *lb = Lb + w.k0 * row + w.c;        // links of the slice before
+                typename PK::Raw *pb = (typename PK::Raw *)pktB + gbase + w.c + w.k0 * V;
+                T before = vb[-RS];
 #pragma unroll
-            for (int u = 0; u < un.value; ++u) {
-                const int s = s0 + u * nthr;
-                const int tl = (int)fd_div((uint32_t)s, f_row), r = s - tl * row;
-                const int e = s + P + 2 * P * tl;
-                const T y = fma(Lb[s], v[e], fma(-h, hop(v + RS, e, s), v[RS + e]));
-                Tb[e] = y;
-                if (cg) acc = fma(y, y, acc);
-                if (tl == 0 || r < P || r >= row - P) PK::store((typename PK::Raw *)pktB + gbase + s + tl * gstep, y, ph);
+                for (int u = 0; u < kSlices; ++u) {
+                    if (u >= w.n) break;
+                    const T here = *vb;
+                    const T y = fma(*lb, before, fma(-h, item_hop(vb, w), here));
+                    *tb = y;
+                    acc = fma(y, y, acc);
+                    if (w.edge || w.k0 + u == 0) PK::store(pb, y, ph);
+                    before = here;
+                    vb += RS;
+                    tb += RS;
+                    lb += row;
+                    pb += V;
+                }
             }
-        });
+        } else {
+            sites([&](int s0, auto un) {
+#pragma unroll
+                for (int u = 0; u < un.value; ++u) {
+                    const int s = s0 + u * nthr;
+                    const int tl = (int)fd_div((uint32_t)s, f_row), r = s - tl * row;
+                    const int e = s + P + 2 * P * tl;
+                    const T y = fma(Lb[s], v[e], fma(-h, hop(v + RS, e, r), v[RS + e]));
+                    Tb[e] = y;
+                    if (cg) acc = fma(y, y, acc);
+                    if (tl == 0 || r < P || r >= row - P) PK::store((typename PK::Raw *)pktB + gbase + s + tl * gstep, y, ph);
+                }
+            });
+        }
         if (cg) {
             par ^= 1;
             publish(acc);
@@ -551,7 +693,7 @@ size_t oc_smem(int d, long long P, int so, int st, bool mixed, bool cheb, bool x
 {
     const long long C = P * so * st, E = P * (so + 2) * (st + 1), Lk = P * so * (st + 1);
     const long long vals = 3 * E + Lk + (x_global ? 0 : C) + (cheb ? 2 * C : 0);
-    return (size_t)(vals * (mixed ? 4 : 8) + (d == 3 ? C : 0) + 16);
+    return (size_t)(vals * (mixed ? 4 : 8) + (d == 3 ? P * so : 0) + 16);
 }
 
 }  // namespace
@@ -634,20 +776,25 @@ OcPlan oc_plan(int d, int nx, int ntau, int nsys, bool mixed, bool cheb, int nsm
                         if (!cols_candidate(d, P, nx, go, so, st, mixed, cheb, &K, &sides, &thr)) continue;
                         sm = oc_cols_smem(d, mixed, cheb, K, thr);
                         const double warps = (thr - 32) / 32;
-                        cost = 7000.0 + 20.0 * go * gt + (sides == 2 ? 2500.0 : 0.0) + (cheb && K > 2 ? 1500.0 : 0.0) +
-                               (!mixed && K == 8 ? 2500.0 : 0.0) +
+                        cost = (mixed ? 5000.0 : 7000.0) + 20.0 * go * gt + (sides == 2 ? 2500.0 : 0.0) + (cheb && K > 2 ? 1500.0 : 0.0) +
+                               (K == 8 ? (mixed ? 1500.0 : 2500.0) : 0.0) +
                                (mixed ? 300.0 : 500.0) * st +
-                               m * (warps * st * (mixed ? 22.0 * d : 16.0 * (d == 1 ? 12 : 20)) + 0.5 * H);
+                               m * (warps * st * (mixed ? 30.0 : 16.0 * (d == 1 ? 12 : 20)) + 0.5 * H);
                     } else {
                         sm = oc_smem(d, P, so, st, mixed, cheb, form == 2);
-                        thr = (int)((C + 31) / 32 * 32);
-                        // More than 8 warps only lengthen the block's barriers and sums while
-                        // a thread has few sites.
-                        if (thr > 256 && C <= 2048) thr = 256;
-                        if (thr > max_threads) thr = max_threads;
+                        // FP32: a thread per item of 4 slices.  FP64: more than 8 warps only lengthen
+                        // the block's barriers while a thread has few sites.
+                        const long long items = mixed ? P * so * ((st + 3) / 4) : C;
+                        thr = items < max_threads ? (int)((items + 31) / 32 * 32) : max_threads;
+                        if (!mixed && thr > 256 && C <= 2048) thr = 256;
                         if (thr < 64) thr = 64;
-                        const double site = mixed ? 2.6 : d == 1 ? 6.5 : 13.0;
-                        cost = 9500.0 + 20.0 * go * gt + m * (C * (site + (form == 2 ? 0.5 : 0.0)) + 0.7 * H);
+                        if (mixed) {
+                            cost = 2600.0 + 20.0 * go * gt + m * (1.6 * C + 1.6 * items + 0.7 * H);
+                            if (cost < 11000.0) cost = 11000.0;
+                        } else {
+                            cost = 9500.0 + 20.0 * go * gt + m * ((d == 1 ? 6.5 : 13.0) * C + 0.7 * H);
+                        }
+                        if (form == 2) cost += 0.5 * m * C;
                     }
                     if (sm > kOcMaxSmem || sm + kStatic > smem_blk || (sm + kStatic) * m > smem_sm) continue;
                     if (best.ok && cost >= best_cost) continue;

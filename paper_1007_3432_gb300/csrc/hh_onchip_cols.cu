@@ -20,8 +20,8 @@
 // FP64 4.4, 4.8 (11.3), mixed 3.6, 4.0 (9.6); 731 x 96 mixed 4.4, 5.8 (11.2);
 // 1024 x 128 mixed 5.2, 6.0 (10.7); d = 3 8^3 x 40 FP64 6.3, 7.0 (17.0);
 // 12^3 x 64 mixed 4.8, 7.0 (15.0).  The tile form stays for tiles that do not fit
-// (wider rows, more slices than registers) and where it is as fast: 16^3 x 64
-// mixed, one right-hand side, 8.2 against 8.5.
+// (wider rows, more slices than registers) and where it is faster: 16^3 x 64
+// mixed, one right-hand side, 6.9 against 8.5.
 #include "hh_onchip_dev.cuh"
 
 namespace hh {
