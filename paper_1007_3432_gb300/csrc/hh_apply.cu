@@ -20,11 +20,12 @@ namespace hh {
 namespace {
 
 // ---------------------------------------------------------------------------
-// Two-sweep path: y = M x (TRANS = false) or y = M^T x (TRANS = true).
+// Two-sweep path: y = M x (TRANS = false) or y = M^T x (TRANS = true), for
+// gridDim.y vectors N sites apart that share the links.
 // ---------------------------------------------------------------------------
 template <int D, typename T, int W, bool TRANS>
 __global__ void __launch_bounds__(256) k_apply_group(const Geo g, const T h, const T *__restrict__ L,
-                                                     const T *__restrict__ x, T *__restrict__ y)
+                                                     const T *__restrict__ x0, T *__restrict__ y0)
 {
     // Programmatic dependent launch: a sweep launched after this one with
     // programmatic stream serialization may start its blocks once every block
@@ -34,6 +35,8 @@ __global__ void __launch_bounds__(256) k_apply_group(const Geo g, const T h, con
     asm volatile("griddepcontrol.launch_dependents;");
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const int stride = W * gridDim.x * blockDim.x;
+    const T *__restrict__ x = x0 + (size_t)blockIdx.y * g.N;
+    T *__restrict__ y = y0 + (size_t)blockIdx.y * g.N;
     for (int i = W * (blockIdx.x * blockDim.x + threadIdx.x); i < g.N; i += stride) {
         GroupNbr nb;
         group_nbrs<D, W>(g, i, nb);
@@ -49,7 +52,7 @@ __global__ void __launch_bounds__(256) k_apply_group(const Geo g, const T h, con
 }
 
 template <typename K, typename T>
-cudaError_t launch_group_kernel(K kern, int blocks, bool pdl, cudaStream_t st, const Geo &g, T h, const T *L,
+cudaError_t launch_group_kernel(K kern, dim3 blocks, bool pdl, cudaStream_t st, const Geo &g, T h, const T *L,
                                 const T *x, T *y)
 {
     if (!pdl) {
@@ -57,7 +60,7 @@ cudaError_t launch_group_kernel(K kern, int blocks, bool pdl, cudaStream_t st, c
         return cudaGetLastError();
     }
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(blocks);
+    cfg.gridDim = blocks;
     cfg.blockDim = dim3(256);
     cfg.dynamicSmemBytes = 0;
     cfg.stream = st;
@@ -70,7 +73,7 @@ cudaError_t launch_group_kernel(K kern, int blocks, bool pdl, cudaStream_t st, c
 }
 
 template <typename T, bool TRANS>
-cudaError_t launch_sweep(const Geo &g, T h, const T *L, const T *x, T *y, cudaStream_t st, bool pdl)
+cudaError_t launch_sweep(const Geo &g, T h, const T *L, const T *x, T *y, cudaStream_t st, bool pdl, int nvec)
 {
     const int w = engine_group_width(g.nx);
     long long groups = g.N / w;
@@ -81,10 +84,10 @@ cudaError_t launch_sweep(const Geo &g, T h, const T *L, const T *x, T *y, cudaSt
         const char *env = getenv("HH_APPLY_SWEEP_BLOCKS");
         return env ? atoi(env) : 152 * 16;
     }();
-    if (cap > 0 && blocks > cap) blocks = cap;
+    if (cap > 0 && blocks > (cap + nvec - 1) / nvec) blocks = (cap + nvec - 1) / nvec;
     if (blocks < 1) blocks = 1;
 #define HH_SWEEP(D, W) \
-    return launch_group_kernel(k_apply_group<D, T, W, TRANS>, blocks, pdl, st, g, h, L, x, y)
+    return launch_group_kernel(k_apply_group<D, T, W, TRANS>, dim3(blocks, nvec), pdl, st, g, h, L, x, y)
     if (g.d == 3) {
         if (w == 4) HH_SWEEP(3, 4);
         else if (w == 2) HH_SWEEP(3, 2);
@@ -294,17 +297,17 @@ cudaError_t launch_mtm_fused_f32(const Geo &g, float h, const float *L, const fl
 }
 
 cudaError_t launch_sweep_f64(const Geo &g, bool trans, double h, const double *L, const double *x, double *y,
-                             cudaStream_t st, bool pdl)
+                             cudaStream_t st, bool pdl, int nvec)
 {
-    return trans ? launch_sweep<double, true>(g, h, L, x, y, st, pdl)
-                 : launch_sweep<double, false>(g, h, L, x, y, st, pdl);
+    return trans ? launch_sweep<double, true>(g, h, L, x, y, st, pdl, nvec)
+                 : launch_sweep<double, false>(g, h, L, x, y, st, pdl, nvec);
 }
 
 cudaError_t launch_sweep_f32(const Geo &g, bool trans, float h, const float *L, const float *x, float *y,
-                             cudaStream_t st, bool pdl)
+                             cudaStream_t st, bool pdl, int nvec)
 {
-    return trans ? launch_sweep<float, true>(g, h, L, x, y, st, pdl)
-                 : launch_sweep<float, false>(g, h, L, x, y, st, pdl);
+    return trans ? launch_sweep<float, true>(g, h, L, x, y, st, pdl, nvec)
+                 : launch_sweep<float, false>(g, h, L, x, y, st, pdl, nvec);
 }
 
 }  // namespace hh

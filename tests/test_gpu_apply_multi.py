@@ -9,7 +9,7 @@ float4 groups divides a warp, else from shared memory); the shapes below
 cover every form, both halo forms, slabs that wrap onto themselves (Nx = 4,
 8), short and odd N_tau (uneven ranges per CTA, ranges that cross from one
 vector to the next), and the full 32^3 x 128 lattice.  Other operators, dtypes and lattices go
-through one hh_apply per vector.  Tolerance as for the single applies:
+through sweeps over groups of vectors, or one hh_apply per vector.  Tolerance as for the single applies:
 |y - y_ref|_i <= 2e-6 (|M| |x|)_i in FP32, 1e-12 in FP64.
 """
 import numpy as np
