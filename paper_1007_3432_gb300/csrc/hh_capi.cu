@@ -243,7 +243,7 @@ size_t oc_packets(const hh_ctx *c, int n_rhs)
 // The forms of the on-chip engine a context uses (decided when it is created).
 int oc_allowed(const hh_ctx *c)
 {
-    if (c->prm.link_order != 0 || c->l16_mode != 0) return 0;
+    if (c->prm.link_order > 1 || c->l16_mode != 0) return 0;
     // An explicit choice of the grid engine's form is a choice of that engine.
     for (const char *name : {"HH_ENGINE_SLOTS", "HH_ENGINE_OVERLAP", "HH_ENGINE_CTL_WARPS",
                              "HH_ENGINE_BLOCKS_PER_SM", "HH_ENGINE_PREFETCH"})
@@ -260,7 +260,8 @@ OcPlan ctx_oc_plan(hh_ctx *c, int n_rhs)
     if (c->oc_forms <= 0) return none;
     if (!c->oc_known[n_rhs]) {
         const bool mixed = c->prm.precision != HH_FP64;
-        c->oc_plans[n_rhs] = oc_plan(c->lat.d, c->lat.nx, c->lat.ntau, n_rhs, mixed, c->prm.cheb_degree > 0, c->nsm,
+        c->oc_plans[n_rhs] = oc_plan(c->lat.d, c->lat.nx, c->lat.ntau, n_rhs, mixed, c->prm.cheb_degree > 0,
+                                     c->prm.link_order == 1, c->nsm,
                                      (size_t)c->smem_sm, (size_t)c->smem_blk, c->oc_forms);
         c->oc_known[n_rhs] = true;
     }

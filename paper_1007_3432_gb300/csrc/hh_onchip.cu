@@ -700,11 +700,11 @@ size_t oc_smem(int d, long long P, int so, int st, bool mixed, bool cheb, bool x
 
 // Column form: a tile's row of so P sites, one per thread, st slices each, with
 // one halo column per edge thread, or two when tiles have one o position (d = 3).
-static bool cols_candidate(int d, long long P, int nx, int go, int so, int st, bool mixed, bool cheb, int *K,
+static bool cols_candidate(int d, long long P, int nx, int go, int so, int st, bool mixed, bool cheb, bool ex, int *K,
                            int *sides, int *threads)
 {
     const long long row = P * so;
-    if (row > kColMaxRow || st > (cheb ? 4 : 8)) return false;
+    if (row > kColMaxRow || st > (cheb || ex ? 4 : 8)) return false;
     *sides = nx / go >= 2 ? 1 : 2;
     if (*sides == 2 && (d == 1 || so != 1)) return false;
     *K = st <= 2 ? 2 : st <= 4 ? 4 : 8;
@@ -714,15 +714,15 @@ static bool cols_candidate(int d, long long P, int nx, int go, int so, int st, b
 
 static const void *plan_kernel(const OcPlan &P, int d)
 {
-    return P.cols ? oc_cols_kernel(d, P.mixed != 0, P.cheb != 0, P.cols, P.sides) : oc_kernel(d, P.mixed != 0, P.cheb != 0);
+    return P.cols ? oc_cols_kernel(d, P.mixed != 0, P.cheb != 0, P.ex != 0, P.cols, P.sides) : oc_kernel(d, P.mixed != 0, P.cheb != 0);
 }
 
 // Registers per thread of a layout's kernel, asked once per process.
 static int kernel_regs(const OcPlan &P, int d)
 {
-    static std::atomic<int> known[2 * 2 * 2 * 3 * 9];
+    static std::atomic<int> known[2 * 2 * 2 * 2 * 3 * 9];
     std::atomic<int> &k =
-        known[(((d == 3) * 2 + (P.mixed != 0)) * 2 + (P.cheb != 0)) * 27 + P.sides * 9 + P.cols];
+        known[((((d == 3) * 2 + (P.mixed != 0)) * 2 + (P.cheb != 0)) * 2 + (P.ex != 0)) * 27 + P.sides * 9 + P.cols];
     int r = k.load(std::memory_order_relaxed);
     if (r == 0) {
         cudaFuncAttributes a;
@@ -746,7 +746,7 @@ int oc_max_blocks(const OcPlan &P, int d)
     return per;
 }
 
-OcPlan oc_plan(int d, int nx, int ntau, int nsys, bool mixed, bool cheb, int nsm, size_t smem_sm, size_t smem_blk,
+OcPlan oc_plan(int d, int nx, int ntau, int nsys, bool mixed, bool cheb, bool ex, int nsm, size_t smem_sm, size_t smem_blk,
                int forms)
 {
     OcPlan best = {};
@@ -765,7 +765,7 @@ OcPlan oc_plan(int d, int nx, int ntau, int nsys, bool mixed, bool cheb, int nsm
                 gt = (ntau + st - 1) / st;
                 if ((long long)go * gt > G) continue;
                 const long long C = P * so * st, H = P * (2 * st + so);
-                for (int form = forms == 2 ? 1 : 0; form < (forms == 3 ? 1 : 3); ++form) {
+                for (int form = forms == 2 ? 1 : 0; form < (forms == 3 || ex ? 1 : 3); ++form) {
                     // form 0: columns; 1, 2: tile form with x in shared or global memory
                     int K = 0, sides = 1, thr = 0;
                     size_t sm;
@@ -773,8 +773,8 @@ OcPlan oc_plan(int d, int nx, int ntau, int nsys, bool mixed, bool cheb, int nsm
                     // st and m on the lattices of the size range (within about 10% of them).
                     double cost;
                     if (form == 0) {
-                        if (!cols_candidate(d, P, nx, go, so, st, mixed, cheb, &K, &sides, &thr)) continue;
-                        sm = oc_cols_smem(d, mixed, cheb, K, thr);
+                        if (!cols_candidate(d, P, nx, go, so, st, mixed, cheb, ex, &K, &sides, &thr)) continue;
+                        sm = oc_cols_smem(d, mixed, cheb, ex, K, thr);
                         const double warps = (thr - 32) / 32;
                         cost = (mixed ? 5000.0 : 7000.0) + 20.0 * go * gt + (sides == 2 ? 2500.0 : 0.0) + (cheb && K > 2 ? 1500.0 : 0.0) +
                                (K == 8 ? (mixed ? 1500.0 : 2500.0) : 0.0) +
@@ -807,6 +807,7 @@ OcPlan oc_plan(int d, int nx, int ntau, int nsys, bool mixed, bool cheb, int nsm
                     p.x_global = form == 2;
                     p.mixed = mixed;
                     p.cheb = cheb;
+                    p.ex = ex;
                     p.cols = K;
                     p.sides = sides;
                     p.smem = sm;

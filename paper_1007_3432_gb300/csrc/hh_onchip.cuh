@@ -24,6 +24,7 @@ struct OcPlan {
     int threads;
     int x_global;       // x stays in global memory (read and written by its owner only)
     int mixed, cheb;
+    int ex;             // exact-block form of M, first order (column form only)
     int cols;           // column form (hh_onchip_cols.cu): slices per thread at most; 0: tile form
     int sides;          // its halo columns per thread: 2 when a tile can have one o position
     size_t smem;        // dynamic shared memory per block
@@ -56,8 +57,8 @@ constexpr int col_max_threads(size_t elem, int K)
 {
     return elem == 8 && K == 8 ? 288 : kColMaxThreads;
 }
-const void *oc_cols_kernel(int d, bool mixed, bool cheb, int K, int sides);
-size_t oc_cols_smem(int d, bool mixed, bool cheb, int K, int threads);
+const void *oc_cols_kernel(int d, bool mixed, bool cheb, bool ex, int K, int sides);
+size_t oc_cols_smem(int d, bool mixed, bool cheb, bool ex, int K, int threads);
 
 // Packet bytes per site and vector, and partial-sum packets per system.
 inline size_t oc_packet_bytes(bool mixed) { return mixed ? 8 : 16; }
@@ -67,7 +68,7 @@ constexpr int kOcReplicas = 8;
 // Layout for nsys systems, on nsm SMs with smem_sm bytes of shared memory per
 // SM and smem_blk at most per block.  forms: 1 the faster form, 2 the tile form,
 // 3 the column form only.
-OcPlan oc_plan(int d, int nx, int ntau, int nsys, bool mixed, bool cheb, int nsm, size_t smem_sm, size_t smem_blk,
+OcPlan oc_plan(int d, int nx, int ntau, int nsys, bool mixed, bool cheb, bool ex, int nsm, size_t smem_sm, size_t smem_blk,
                int forms);
 
 // Blocks of a layout's kernel that one SM holds at once.

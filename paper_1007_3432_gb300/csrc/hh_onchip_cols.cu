@@ -21,7 +21,9 @@
 // 1024 x 128 mixed 5.2, 6.0 (10.7); d = 3 8^3 x 40 FP64 6.3, 7.0 (17.0);
 // 12^3 x 64 mixed 4.8, 7.0 (15.0).  The tile form stays for tiles that do not fit
 // (wider rows, more slices than registers) and where it is faster: 16^3 x 64
-// mixed, one right-hand side, 6.9 against 8.5.
+// mixed, one right-hand side, 6.9 against 8.5.  The exact-block form of M to first
+// order exists in this form only: observables on 10^3 x 48 FP64, 4 noise vectors,
+// 38.6 ms on the grid engine (scalar loops that recompute the hops), 21.8 here.
 #include "hh_onchip_dev.cuh"
 
 namespace hh {
@@ -241,7 +243,11 @@ __device__ __forceinline__ uint32_t control_warp(const OcLaunch &L, ColShared<T>
 }
 
 // The compute warps: thread c of them owns the spatial site c of the tile's row.
-template <int D, typename T, int K, int SIDES, bool CHEB>
+// EX: the exact-block form of M to first order (link_order 1),
+//   (M v)(tau) = v(tau) + (1 + h H) (L v)(tau - 1),  (M^T t)(tau) = t(tau) + L(tau) (1 + h H) t(tau + 1):
+// the hops are on the slice before or after, so staged row k holds L v of slice
+// k - 1, or t of slice k + 1, and the halo columns are those of these slices.
+template <int D, typename T, int K, int SIDES, bool CHEB, bool EX>
 __device__ __forceinline__ void compute_warps(const OcLaunch &L, ColShared<T> &S, unsigned char *smem, int sid, int tile)
 {
     constexpr bool MIXED = sizeof(T) == 4;
@@ -252,6 +258,8 @@ __device__ __forceinline__ void compute_warps(const OcLaunch &L, ColShared<T> &S
     T *const Pb = (T *)smem;                        // p, o halo included: slice k at k RS
     T *const Tb = Pb + K * RS;                      // t
     T *const Wb = CHEB ? Tb + K * RS : Pb;          // preconditioner: M's input there (p stays in Pb)
+    T *const Ph = EX ? Tb + K * RS : Pb;            // EX: p of the halo columns, and their links
+    T *const Lh = EX ? Ph + K * RS : Pb;
     const int tid = (int)threadIdx.x, nthr = (int)blockDim.x, c = tid - 32;
     EngCtl *const ctl = L.ctl;
 
@@ -292,6 +300,13 @@ __device__ __forceinline__ void compute_warps(const OcLaunch &L, ColShared<T> &S
     Raw *const pktA = (Raw *)L.pkt + (size_t)sid * 2 * L.N;
     Raw *p_own = pktA + g0, *p_side = pktA + gs, *p_right = pktA + gr;
     const int d_prev = gp - g0, d_next = gn - g0 + L.N;     // slice before (A) and after (B) from p_own
+    // Halo packet of staged row u, from the halo column's slice 0.
+    const int s_prev = gp - g0, s_next = gn - g0;           // (the same steps as in the own column)
+    auto halo_step = [&](bool after, int u) -> int {
+        if (!EX) return u * V;
+        if (after) return u + 1 < st ? (u + 1) * V : s_next;
+        return u == 0 ? s_prev : (u - 1) * V;
+    };
 
     const T h = (T)Y.h;
     // The preconditioner's M input and z take the registers of p and x, which its
@@ -307,6 +322,12 @@ __device__ __forceinline__ void compute_warps(const OcLaunch &L, ColShared<T> &S
             lk[k] = active && k < st ? __ldg(src + g0 + k * V) : T(0);
         }
         if (active) lkp = __ldg(src + gp);
+        if (EX && side)
+#pragma unroll
+            for (int k = 0; k < SIDES * K; ++k) {
+                const int u = k < K ? k : k - K;
+                if (u < st) Lh[(k < K ? k * RS + hidx : u * RS + row + P + pos)] = __ldg(src + (k < K ? gs : gr) + halo_step(false, u));
+            }
     }
     uint32_t ph = (uint32_t)L.seq[0];
 
@@ -340,7 +361,9 @@ __device__ __forceinline__ void compute_warps(const OcLaunch &L, ColShared<T> &S
         constexpr int B = MIXED || U <= 5 ? U : 5;
         keep_base();
         auto where = [&](int u) -> const Raw * {
-            return u == U - 1 ? p_own + d_time : u < K ? p_side + off + u * V : p_right + off + (u - K) * V;
+            return u == U - 1 ? p_own + d_time
+                   : u < K   ? p_side + off + halo_step(off != 0, u)
+                             : p_right + off + halo_step(off != 0, u - K);
         };
         auto wanted = [&](int u) -> bool { return u == U - 1 ? active : side && (u < K ? u : u - K) < st; };
         SpinClock clk;
@@ -397,6 +420,7 @@ __device__ __forceinline__ void compute_warps(const OcLaunch &L, ColShared<T> &S
     // (M^T t) at slice k.
     auto mt = [&](int k) -> T {
         const T nv = k + 1 < K && k + 1 < st ? t[k + 1 < K ? k + 1 : k] : tv;
+        if (EX) return fma(lk[k], fma(h, hop(Tb + k * RS), nv), t[k]);
         return fma(lk[k], nv, fma(-h, hop(Tb + k * RS), t[k]));
     };
 
@@ -409,7 +433,10 @@ __device__ __forceinline__ void compute_warps(const OcLaunch &L, ColShared<T> &S
         bool bad = false;
         if (pm != MODE_NEW) {
             bad = !fetch_halo(stageB ? L.N : 0, stageB ? d_next : d_prev);
-            if (stageB) stage_halo(Tb, false, T(0));
+            if (stageB) {
+                stage_halo(Tb, false, T(0));
+                if (EX && active) Tb[(st - 1) * RS + me] = tv;
+            }
         }
         if (bar_all(nthr, bad)) break;
 
@@ -530,7 +557,8 @@ __device__ __forceinline__ void compute_warps(const OcLaunch &L, ColShared<T> &S
                     const int g = g0 + k * V;
                     Nbr nb;
                     neighbours(Y.g, g, nb);
-                    Y.t[g] = stencil_M<double>(Y.g, Y.h, Y.L64, Y.x, g, nb);
+                    Y.t[g] = EX ? stencil_M_ex<double>(Y.g, Y.h, Y.L64, Y.x, g, nb, 1)
+                                : stencil_M<double>(Y.g, Y.h, Y.L64, Y.x, g, nb);
                 }
             if (tile_barrier()) break;
             ++ph;
@@ -542,7 +570,9 @@ __device__ __forceinline__ void compute_warps(const OcLaunch &L, ColShared<T> &S
                     const int g = g0 + k * V;
                     Nbr nb;
                     neighbours(Y.g, g, nb);
-                    const double res = __ldg(Y.b + g) - stencil_MT<double>(Y.g, Y.h, Y.L64, Y.t, g, nb);
+                    const double res =
+                        __ldg(Y.b + g) - (EX ? stencil_MT_ex<double>(Y.g, Y.h, Y.L64, Y.t, g, nb, 1)
+                                             : stencil_MT<double>(Y.g, Y.h, Y.L64, Y.t, g, nb));
                     acc = fma(res, res, acc);
                     if (MIXED) Y.r[g] = res;
                     Tb[k * RS + me] = (T)res;     // to the registers below (staged t is not read any more)
@@ -585,8 +615,14 @@ __device__ __forceinline__ void compute_warps(const OcLaunch &L, ColShared<T> &S
                 for (int k = 0; k < K; ++k) pw[k] = restart ? r[k] : fma(beta, pw[k], r[k]);
             }
             vp = pp = restart ? tv : fma(beta, pp, tv);
-            // The halo of p is kept where it is staged.
-            stage_halo(Pb, !restart, beta);
+            // The halo of p is kept where it is staged (EX: L p is staged).
+            stage_halo(EX ? Ph : Pb, !restart, beta);
+            if (EX && side)
+#pragma unroll
+                for (int k = 0; k < SIDES * K; ++k) {
+                    const int u = k < K ? k : k - K, cell = k < K ? k * RS + hidx : u * RS + row + P + pos;
+                    if (u < st) Pb[cell] = Lh[cell] * Ph[cell];
+                }
         } else {
             stage_halo(Wb, false, T(0));
         }
@@ -594,7 +630,7 @@ __device__ __forceinline__ void compute_warps(const OcLaunch &L, ColShared<T> &S
         if (active) {
 #pragma unroll
             for (int k = 0; k < K; ++k)
-                if (k < st) Sb[k * RS + me] = v_of(k);
+                if (k < st) Sb[k * RS + me] = !EX ? v_of(k) : k == 0 ? lkp * vp : lk[k > 0 ? k - 1 : 0] * v_of(k > 0 ? k - 1 : 0);
         }
         bar_sync(kBarStage, nthr - 32);
         T acc = T(0);
@@ -604,9 +640,15 @@ __device__ __forceinline__ void compute_warps(const OcLaunch &L, ColShared<T> &S
                 if (k < st) {
                     const T vm = k == 0 ? vp : v_of(k > 0 ? k - 1 : 0);
                     const T lm = k == 0 ? lkp : lk[k > 0 ? k - 1 : 0];
-                    t[k] = fma(lm, vm, fma(-h, hop(Sb + k * RS), v_of(k)));
+                    if (EX)
+                        t[k] = v_of(k) + fma(h, hop(Sb + k * RS), lm * vm);
+                    else
+                        t[k] = fma(lm, vm, fma(-h, hop(Sb + k * RS), v_of(k)));
                     acc = fma(t[k], t[k], acc);
-                    Tb[k * RS + me] = t[k];
+                    if (!EX)
+                        Tb[k * RS + me] = t[k];
+                    else if (k > 0)
+                        Tb[(k - 1) * RS + me] = t[k];
                     if (side || k == 0) PK::store(p_own + L.N + k * V, t[k], ph);
                 }
         }
@@ -620,7 +662,7 @@ __device__ __forceinline__ void compute_warps(const OcLaunch &L, ColShared<T> &S
     }
 }
 
-template <int D, typename T, int K, int SIDES, bool CHEB>
+template <int D, typename T, int K, int SIDES, bool CHEB, bool EX = false>
 __global__ void __launch_bounds__(col_max_threads(sizeof(T), K), 1) k_onchip_cols(const OcLaunch L)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -638,7 +680,7 @@ __global__ void __launch_bounds__(col_max_threads(sizeof(T), K), 1) k_onchip_col
     }
     __syncthreads();
     if (tid >= 32) {
-        compute_warps<D, T, K, SIDES, CHEB>(L, S, smem, sid, tile);
+        compute_warps<D, T, K, SIDES, CHEB, EX>(L, S, smem, sid, tile);
         return;
     }
     const uint32_t phases = control_warp<T, CHEB>(L, S, sid, tile);
@@ -653,8 +695,14 @@ __global__ void __launch_bounds__(col_max_threads(sizeof(T), K), 1) k_onchip_col
 }
 
 template <int D, int SIDES>
-const void *cols_kernel_d(bool mixed, bool cheb, int K)
+const void *cols_kernel_d(bool mixed, bool cheb, bool ex, int K)
 {
+    if (ex) {
+        if (mixed) return K <= 2 ? (const void *)k_onchip_cols<D, float, 2, SIDES, false, true>
+                                 : (const void *)k_onchip_cols<D, float, 4, SIDES, false, true>;
+        return K <= 2 ? (const void *)k_onchip_cols<D, double, 2, SIDES, false, true>
+                      : (const void *)k_onchip_cols<D, double, 4, SIDES, false, true>;
+    }
     if (mixed) {
         if (K <= 2) return (const void *)k_onchip_cols<D, float, 2, SIDES, false>;
         if (K <= 4) return (const void *)k_onchip_cols<D, float, 4, SIDES, false>;
@@ -671,16 +719,16 @@ const void *cols_kernel_d(bool mixed, bool cheb, int K)
 
 }  // namespace
 
-const void *oc_cols_kernel(int d, bool mixed, bool cheb, int K, int sides)
+const void *oc_cols_kernel(int d, bool mixed, bool cheb, bool ex, int K, int sides)
 {
-    if (d == 1) return cols_kernel_d<1, 1>(mixed, cheb, K);
-    return sides == 1 ? cols_kernel_d<3, 1>(mixed, cheb, K) : cols_kernel_d<3, 2>(mixed, cheb, K);
+    if (d == 1) return cols_kernel_d<1, 1>(mixed, cheb, ex, K);
+    return sides == 1 ? cols_kernel_d<3, 1>(mixed, cheb, ex, K) : cols_kernel_d<3, 2>(mixed, cheb, ex, K);
 }
 
-size_t oc_cols_smem(int d, bool mixed, bool cheb, int K, int threads)
+size_t oc_cols_smem(int d, bool mixed, bool cheb, bool ex, int K, int threads)
 {
     const size_t rs = d == 1 ? kColStride<1> : kColStride<3>;
-    return K * ((cheb ? 3 : 2) * rs + (cheb ? (size_t)(threads - 32) : 0)) * (mixed ? 4 : 8);
+    return K * ((cheb ? 3 : ex ? 4 : 2) * rs + (cheb ? (size_t)(threads - 32) : 0)) * (mixed ? 4 : 8);
 }
 
 }  // namespace hh

@@ -157,3 +157,25 @@ def test_onchip_layouts_alternate_in_one_context(hh, monkeypatch):
         ctx.set_field(sigma)
         for k in (1, 3, 2, 1, 1, 3):
             assert torch.equal(one(ctx, k), fresh[k])
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("d,nx,ntau", [(1, 2, 2), (1, 2, 5), (1, 33, 9), (1, 500, 7), (3, 2, 3), (3, 3, 5), (3, 5, 16),
+                                       (3, 10, 12), (3, 16, 6)])
+@pytest.mark.parametrize("n_rhs", [1, 3])
+def test_onchip_exact_block_first_order(hh, monkeypatch, d, nx, ntau, precision, n_rhs):
+    """The exact-block form to first order: its halos are those of the slice
+    before and after (corners of the tiles included)."""
+    n = nx ** d * ntau
+    sigma = workloads.sigma_field(n, seed=2000 + nx + ntau)
+    b = np.stack([workloads.source(n, seed=2001, rhs=a) for a in range(n_rhs)])
+    rc, info, x, cnt = _solve(hh, monkeypatch, 1, d, nx, ntau, precision, b, sigma, link_order=1)
+    rc0, info0, x0, _ = _solve(hh, monkeypatch, 0, d, nx, ntau, precision, b, sigma, link_order=1)
+    assert rc == 0 and rc0 == 0 and info["converged"] == 1 and info["true_relres"] <= 1e-10
+    lat = oracle.lattice(d, nx, ntau)
+    L = oracle.links(lat, A, sigma)
+    for a in range(n_rhs):
+        res = b[a] - oracle.apply_MTM_ex(lat, H, L, 1, x[a])
+        assert np.linalg.norm(res) <= 1.0001e-10 * np.linalg.norm(b[a])
+    assert abs(info["iterations"] - info0["iterations"]) <= 2 + 0.03 * info0["iterations"], (info, info0)
+    assert np.linalg.norm(x - x0) <= 1e-4 * np.linalg.norm(x0)
