@@ -159,6 +159,8 @@ struct hh_ctx {
     ulonglong2 *d_slots;
     unsigned long long *d_seq;
     int oc_cap, oc_last;
+    void *oc_old[65];       // blocks that a larger one has replaced: a captured solve may be
+    int n_oc_old;           // replayed on them, so they live as long as the context
     int oc_forms;           // on-chip engine: 0 not used, 1 by rule, 2 tile form, 3 column form only
     bool oc_known[65];      // layouts by number of systems (n_pf <= 64), once computed
     OcPlan oc_plans[65];
@@ -227,6 +229,7 @@ void free_ctx(hh_ctx *c)
         if (p) cudaFree(p);
     if (c->L16) cudaFree(c->L16);
     if (c->d_slots) cudaFree(c->d_slots);    // d_seq and d_pkt lie behind it
+    for (int i = 0; i < c->n_oc_old; ++i) cudaFree(c->oc_old[i]);
     if (c->ev) {
         for (int i = 0; i < c->ev_cap; ++i)
             if (c->ev[i]) cudaEventDestroy(c->ev[i]);
@@ -276,7 +279,7 @@ OcPlan ctx_oc_plan(hh_ctx *c, int n_rhs)
             cudaGetLastError();
             return none;
         }
-        if (c->d_slots) cudaFree(c->d_slots);    // waits for the work that uses it
+        if (c->d_slots) c->oc_old[c->n_oc_old++] = c->d_slots;
         c->d_slots = (ulonglong2 *)blk;
         c->d_seq = (unsigned long long *)(blk + sb);
         c->d_pkt = blk + sb + 256;

@@ -22,7 +22,8 @@
 // is next written after its block has read the t packets (phase n + 1) of the
 // sites around it, and those were published after their blocks had read the r
 // packet; likewise for t, and for partial sums, whose two parities
-// alternate.  The reliable update exchanges x and t in global memory between
+// alternate.  (Where a phase ends in a sum, the sum alone orders them: every tile
+// has read the packets of the phase before it gives its part.)  The reliable update exchanges x and t in global memory between
 // barriers made of the same sums with fences around them.
 //
 // What bounds it: the chain exchange - barrier - phase - block sum, run by a few
@@ -714,7 +715,8 @@ static bool cols_candidate(int d, long long P, int nx, int go, int so, int st, b
 
 static const void *plan_kernel(const OcPlan &P, int d)
 {
-    return P.cols ? oc_cols_kernel(d, P.mixed != 0, P.cheb != 0, P.ex != 0, P.cols, P.sides) : oc_kernel(d, P.mixed != 0, P.cheb != 0);
+    if (P.cols) return oc_cols_kernel(d, P.mixed != 0, P.cheb != 0, P.ex != 0, P.cols, P.sides);
+    return oc_kernel(d, P.mixed != 0, P.cheb != 0);
 }
 
 // Registers per thread of a layout's kernel, asked once per process.
@@ -776,8 +778,8 @@ OcPlan oc_plan(int d, int nx, int ntau, int nsys, bool mixed, bool cheb, bool ex
                         if (!cols_candidate(d, P, nx, go, so, st, mixed, cheb, ex, &K, &sides, &thr)) continue;
                         sm = oc_cols_smem(d, mixed, cheb, ex, K, thr);
                         const double warps = (thr - 32) / 32;
-                        cost = (mixed ? 5000.0 : 7000.0) + 20.0 * go * gt + (sides == 2 ? 2500.0 : 0.0) + (cheb && K > 2 ? 1500.0 : 0.0) +
-                               (K == 8 ? (mixed ? 1500.0 : 2500.0) : 0.0) +
+                        cost = (mixed ? 5000.0 : 7000.0) + 20.0 * go * gt + (sides == 2 ? 2500.0 : 0.0) +
+                               (cheb && K > 2 ? 1500.0 : 0.0) + (K == 8 ? (mixed ? 1500.0 : 2500.0) : 0.0) +
                                (mixed ? 300.0 : 500.0) * st +
                                m * (warps * st * (mixed ? 30.0 : 16.0 * (d == 1 ? 12 : 20)) + 0.5 * H);
                     } else {

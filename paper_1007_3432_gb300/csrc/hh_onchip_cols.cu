@@ -7,8 +7,8 @@
 // are then in the same thread, the row before the tile and the one after it
 // are read from their packets straight into registers, and shared memory only
 // carries the 2d spatial neighbours, at constant strides.  The threads at the
-// tile's o edges fetch and hold the halo columns (hence at least two o
-// positions per tile).  Warp 0 does nothing but wait for sums, decide and
+// tile's o edges fetch the halo columns, one each, or both when the tile has one
+// o position (SIDES).  Warp 0 does nothing but wait for sums, decide and
 // publish; the other warps hand it their partial sums at a barrier they do not
 // wait on.
 //
@@ -38,7 +38,7 @@ constexpr int kColStride = D == 1 ? kColMaxRow + 2 : 3 * kColMaxRow;
 
 // Barriers (the roles run different code, so all of them are numbered ones).
 constexpr int kBarStage = 1;    // compute warps: a vector is staged
-constexpr int kBarSum = 2;      // compute warps arrive, warp 0 waits: partial sums in s_red
+constexpr int kBarSum = 2;      // compute warps arrive, warp 0 waits: partial sums in red
 constexpr int kBarAll = 3;      // the whole block
 
 __device__ __forceinline__ void bar_sync(int id, int n)
