@@ -179,3 +179,32 @@ def test_onchip_exact_block_first_order(hh, monkeypatch, d, nx, ntau, precision,
         assert np.linalg.norm(res) <= 1.0001e-10 * np.linalg.norm(b[a])
     assert abs(info["iterations"] - info0["iterations"]) <= 2 + 0.03 * info0["iterations"], (info, info0)
     assert np.linalg.norm(x - x0) <= 1e-4 * np.linalg.norm(x0)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_onchip_solve_replays_from_a_graph(hh, monkeypatch, precision):
+    """A captured solve goes on from the phase numbers on the device: replays,
+    with a plain solve between them, give the plain solve's bits."""
+    monkeypatch.setenv("HH_ENGINE_ONCHIP", "1")
+    d, nx, ntau = 1, 48, 24
+    n = nx * ntau
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        b = dev(workloads.source(n, seed=2100))
+        x = torch.zeros_like(b)
+        with hh.Context(d, nx, ntau, precision=precision) as ctx:
+            ctx.set_field(dev(workloads.sigma_field(n, seed=2101)))
+            ctx.solve(b, x, 1)
+            ref = x.clone()
+            stream.synchronize()
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=stream):
+                ctx.solve(b, x, 1, info=False)
+            for _ in range(2):
+                x.zero_()
+                g.replay()
+                stream.synchronize()
+                assert torch.equal(x, ref)
+                x.zero_()
+                ctx.solve(b, x, 1)
+                assert torch.equal(x, ref)
