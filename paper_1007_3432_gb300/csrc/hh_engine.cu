@@ -750,8 +750,9 @@ __global__ void __launch_bounds__(ENGINE_BLOCK, MINB) engine_kernel(EngLaunch L)
     __shared__ EngSystem s_sysd[kCacheSys];
 
     EngCtl *ctl = L.ctl;
-    // An error recorded before this launch (by the on-chip engine) ends it.
-    if (ld_volatile_i32(&ctl->error) != 0) return;
+    // An error recorded before this launch (by the on-chip engine) ends it.  Blocks of
+    // this launch write the word too, so one thread's read decides for the block.
+    if (__syncthreads_or(threadIdx.x == 0 && ld_volatile_i32(&ctl->error) != 0)) return;
     const unsigned G = gridDim.x;
     long long k = *(volatile long long *)&ctl->k;
     const int drop = *(volatile int *)&ctl->drop_sig;   // tile partial (+ 1) never published: tests only

@@ -17,7 +17,9 @@ admits no cycle of waits.  It also checks the rule is necessary: publishing
 after the next preparation unconditionally deadlocks on layouts that are not
 homogeneous, and so does a homogeneous layout with a single system.
 """
+import os
 import random
+import re
 
 import pytest
 
@@ -159,3 +161,18 @@ def test_single_system_needs_publish_first():
     layout = [[0], [0], [0]]
     assert not simulate(layout, 1, levels=3, rule="always_delay", rng=random.Random(1))
     assert simulate(layout, 1, levels=3, rule="engine", rng=random.Random(1))
+
+
+def test_early_exit_is_one_decision_of_the_block():
+    """Other blocks of the same launch write EngCtl::error when a wait runs
+    out, so threads of a block that start at different times may read different
+    values: a block that left by a per-thread read would lose part of its
+    threads before its first barrier.  Every return of engine_kernel ahead of
+    that barrier must be taken by all threads or none."""
+    src = os.path.join(os.path.dirname(__file__), "..", "paper_1007_3432_gb300", "csrc", "hh_engine.cu")
+    body = open(src).read().split("engine_kernel(EngLaunch L)", 1)[1]
+    head = body[:body.index("__syncthreads();")]
+    head = re.sub(r"//[^\n]*", "", head)
+    returns = re.findall(r"[^;{}]*\breturn\b", head)
+    assert len(returns) == 1, returns
+    assert re.match(r"\s*if \(__syncthreads_or\(", returns[0]), returns
