@@ -40,6 +40,7 @@
 #include <atomic>
 
 #include "hh_onchip_dev.cuh"
+#include "hh_onchip_plan.cuh"
 
 namespace hh {
 
@@ -673,12 +674,6 @@ __global__ void __launch_bounds__(kOcMaxThreads, 1) k_onchip(const OcLaunch L)
     }
 }
 
-// Dynamic shared memory a block may ask for: the 227 KB a block can have, less
-// the kernels' static part.  The kernels' limit is set to it, whatever a
-// launch uses, so that threads launching different layouts do not race on it.
-constexpr int kOcStaticSmem = 2048;
-constexpr int kOcMaxSmem = 227 * 1024 - kOcStaticSmem;
-
 const void *oc_kernel(int d, bool mixed, bool cheb)
 {
     if (d == 1)
@@ -688,30 +683,7 @@ const void *oc_kernel(int d, bool mixed, bool cheb)
                  : cheb ? (const void *)k_onchip<3, double, true> : (const void *)k_onchip<3, double, false>;
 }
 
-// Dynamic shared memory of a block whose tile is at most so x st columns of P
-// sites (the kernel's layout).
-size_t oc_smem(int d, long long P, int so, int st, bool mixed, bool cheb, bool x_global)
-{
-    const long long C = P * so * st, E = P * (so + 2) * (st + 1), Lk = P * so * (st + 1);
-    const long long vals = 3 * E + Lk + (x_global ? 0 : C) + (cheb ? 2 * C : 0);
-    return (size_t)(vals * (mixed ? 4 : 8) + (d == 3 ? P * so : 0) + 16);
-}
-
 }  // namespace
-
-// Column form: a tile's row of so P sites, one per thread, st slices each, with
-// one halo column per edge thread, or two when tiles have one o position (d = 3).
-static bool cols_candidate(int d, long long P, int nx, int go, int so, int st, bool mixed, bool cheb, bool ex, int *K,
-                           int *sides, int *threads)
-{
-    const long long row = P * so;
-    if (row > kColMaxRow || st > (cheb || ex ? 4 : 8)) return false;
-    *sides = nx / go >= 2 ? 1 : 2;
-    if (*sides == 2 && (d == 1 || so != 1)) return false;
-    *K = st <= 2 ? 2 : st <= 4 ? 4 : 8;
-    *threads = (int)((row + 31) / 32 * 32) + 32;
-    return *threads <= col_max_threads(mixed ? 4 : 8, *K);
-}
 
 static const void *plan_kernel(const OcPlan &P, int d)
 {
@@ -751,80 +723,8 @@ int oc_max_blocks(const OcPlan &P, int d)
 OcPlan oc_plan(int d, int nx, int ntau, int nsys, bool mixed, bool cheb, bool ex, int nsm, size_t smem_sm, size_t smem_blk,
                int forms)
 {
-    OcPlan best = {};
-    const long long P = d == 3 ? (long long)nx * nx : 1;
-    double best_cost = 0.0;
-    constexpr size_t kStatic = kOcStaticSmem;    // static and reserved shared memory per block
-    for (int m = 1; m <= 4; ++m) {
-        const int G = (int)((long long)nsm * m / nsys) < kOcMaxTiles ? nsm * m / nsys : kOcMaxTiles;
-        if (G < 1) continue;
-        const int max_threads = kOcMaxThreads / m;
-        // Tile extents that differ: so = ceil(nx / go), st = ceil(ntau / gt), with the fewest tiles each.
-        for (int go = 1; go <= nx && go <= G; ++go) {
-            const int so = (nx + go - 1) / go;
-            if (go > 1 && (nx + go - 2) / (go - 1) == so) continue;
-            for (int st = 1, gt; st <= ntau; st = gt == 1 ? ntau + 1 : (ntau + gt - 2) / (gt - 1)) {
-                gt = (ntau + st - 1) / st;
-                if ((long long)go * gt > G) continue;
-                const long long C = P * so * st, H = P * (2 * st + so);
-                for (int form = forms == 2 ? 1 : 0; form < (forms == 3 || ex ? 1 : 3); ++form) {
-                    // form 0: columns; 1, 2: tile form with x in shared or global memory
-                    int K = 0, sides = 1, thr = 0;
-                    size_t sm;
-                    // Clocks of one iteration on an SM holding m tiles, from times measured over so,
-                    // st and m on the lattices of the size range (within about 10% of them).
-                    double cost;
-                    if (form == 0) {
-                        if (!cols_candidate(d, P, nx, go, so, st, mixed, cheb, ex, &K, &sides, &thr)) continue;
-                        sm = oc_cols_smem(d, mixed, cheb, ex, K, thr);
-                        const double warps = (thr - 32) / 32;
-                        cost = (mixed ? 5000.0 : 7000.0) + 20.0 * go * gt + (sides == 2 ? 2500.0 : 0.0) +
-                               (cheb && K > 2 ? 1500.0 : 0.0) + (K == 8 ? (mixed ? 1500.0 : 2500.0) : 0.0) +
-                               (mixed ? 300.0 : 500.0) * st +
-                               m * (warps * st * (mixed ? 30.0 : 16.0 * (d == 1 ? 12 : 20)) + 0.5 * H);
-                    } else {
-                        sm = oc_smem(d, P, so, st, mixed, cheb, form == 2);
-                        // FP32: a thread per item of 4 slices.  FP64: more than 8 warps only lengthen
-                        // the block's barriers while a thread has few sites.
-                        const long long items = mixed ? P * so * ((st + 3) / 4) : C;
-                        thr = items < max_threads ? (int)((items + 31) / 32 * 32) : max_threads;
-                        if (!mixed && thr > 256 && C <= 2048) thr = 256;
-                        if (thr < 64) thr = 64;
-                        if (mixed) {
-                            cost = 2600.0 + 20.0 * go * gt + m * (1.6 * C + 1.6 * items + 0.7 * H);
-                            if (cost < 11000.0) cost = 11000.0;
-                        } else {
-                            cost = 9500.0 + 20.0 * go * gt + m * ((d == 1 ? 6.5 : 13.0) * C + 0.7 * H);
-                        }
-                        if (form == 2) cost += 0.5 * m * C;
-                    }
-                    if (sm > kOcMaxSmem || sm + kStatic > smem_blk || (sm + kStatic) * m > smem_sm) continue;
-                    if (best.ok && cost >= best_cost) continue;
-                    OcPlan p = {};
-                    p.ok = 1;
-                    p.go = go;
-                    p.gt = gt;
-                    p.so = so;
-                    p.st = st;
-                    p.x_global = form == 2;
-                    p.mixed = mixed;
-                    p.cheb = cheb;
-                    p.ex = ex;
-                    p.cols = K;
-                    p.sides = sides;
-                    p.smem = sm;
-                    p.threads = thr;
-                    // Co-resident, as its blocks wait on one another: by registers (a
-                    // warp's are one of the 4 partitions', 16384 each) and shared memory.
-                    const int regs = (kernel_regs(p, d) + 7) / 8 * 8;
-                    const int parts = (thr / 32 + 3) / 4;    // warps of a block per partition
-                    if (regs <= 0 || 16384 / (regs * 32) / parts < m) continue;
-                    best_cost = cost;
-                    best = p;
-                }
-            }
-        }
-    }
+    OcPlan best = oc_choose(d, nx, ntau, nsys, mixed, cheb, ex, nsm, smem_sm, smem_blk, forms,
+                            [d](const OcPlan &p) { return kernel_regs(p, d); });
     // The occupancy calculation has the last word.
     if (best.ok && oc_max_blocks(best, d) * nsm < best.go * best.gt * nsys) best.ok = 0;
     return best;
@@ -832,6 +732,7 @@ OcPlan oc_plan(int d, int nx, int ntau, int nsys, bool mixed, bool cheb, bool ex
 
 cudaError_t oc_launch(const OcLaunch &L, const OcPlan &P, int d, cudaStream_t st)
 {
+    if (P.threads % 32 != 0) return cudaErrorInvalidConfiguration;
     const void *fn = plan_kernel(P, d);
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kOcMaxSmem);
     if (e != cudaSuccess) return e;

@@ -58,7 +58,19 @@ constexpr int col_max_threads(size_t elem, int K)
     return elem == 8 && K == 8 ? 288 : kColMaxThreads;
 }
 const void *oc_cols_kernel(int d, bool mixed, bool cheb, bool ex, int K, int sides);
-size_t oc_cols_smem(int d, bool mixed, bool cheb, bool ex, int K, int threads);
+
+// Row stride of the staged vectors, in elements: constant, so that the K rows of
+// a neighbour are one address and immediate offsets.  d = 3: (so + 2) P sites,
+// at most three times the row.
+template <int D>
+constexpr int kColStride = D == 1 ? kColMaxRow + 2 : 3 * kColMaxRow;
+
+// Its dynamic shared memory per block.
+inline size_t oc_cols_smem(int d, bool mixed, bool cheb, bool ex, int K, int threads)
+{
+    const size_t rs = d == 1 ? kColStride<1> : kColStride<3>;
+    return K * ((cheb ? 3 : ex ? 4 : 2) * rs + (cheb ? (size_t)(threads - 32) : 0)) * (mixed ? 4 : 8);
+}
 
 // Packet bytes per site and vector, and partial-sum packets per system.
 inline size_t oc_packet_bytes(bool mixed) { return mixed ? 8 : 16; }

@@ -30,12 +30,6 @@ namespace hh {
 
 namespace {
 
-// Row stride of the staged vectors, in elements: constant, so that the K rows of
-// a neighbour are one address and immediate offsets.  d = 3: (so + 2) P sites,
-// at most three times the row.
-template <int D>
-constexpr int kColStride = D == 1 ? kColMaxRow + 2 : 3 * kColMaxRow;
-
 // Barriers (the roles run different code, so all of them are numbered ones).
 constexpr int kBarStage = 1;    // compute warps: a vector is staged
 constexpr int kBarSum = 2;      // compute warps arrive, warp 0 waits: partial sums in red
@@ -723,12 +717,6 @@ const void *oc_cols_kernel(int d, bool mixed, bool cheb, bool ex, int K, int sid
 {
     if (d == 1) return cols_kernel_d<1, 1>(mixed, cheb, ex, K);
     return sides == 1 ? cols_kernel_d<3, 1>(mixed, cheb, ex, K) : cols_kernel_d<3, 2>(mixed, cheb, ex, K);
-}
-
-size_t oc_cols_smem(int d, bool mixed, bool cheb, bool ex, int K, int threads)
-{
-    const size_t rs = d == 1 ? kColStride<1> : kColStride<3>;
-    return K * ((cheb ? 3 : ex ? 4 : 2) * rs + (cheb ? (size_t)(threads - 32) : 0)) * (mixed ? 4 : 8);
 }
 
 }  // namespace hh

@@ -84,6 +84,18 @@ def test_host_logic_tiling_and_md_schedules(tmp_path):
     assert out.returncode == 0 and out.stdout.strip() == "ok", out.stdout + out.stderr
 
 
+def test_onchip_layout_rule(tmp_path):
+    """Layouts of the on-chip engine: whole warps, tiles that cover the
+    lattice, blocks that fit on the chip at once (host-only build)."""
+    import shutil
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    exe = str(tmp_path / "onchip_plan_check")
+    subprocess.check_call([nvcc, "-O2", "-std=c++17", "-I", os.path.join(ROOT, "include"),
+                           os.path.join(ROOT, "tests", "native", "onchip_plan_check.cu"), "-o", exe])
+    out = subprocess.run([exe], capture_output=True, text=True)
+    assert out.returncode == 0 and out.stdout.strip() == "ok", out.stdout + out.stderr
+
+
 def test_chebyshev_table_matches_oracle_polynomial(tmp_path):
     """The engine's Chebyshev table (Leja-ordered real factors, Sec. 4.2),
     evaluated factor by factor on the host, against the oracle's P(z) of
