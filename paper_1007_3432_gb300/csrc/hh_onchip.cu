@@ -723,11 +723,10 @@ int oc_max_blocks(const OcPlan &P, int d)
 OcPlan oc_plan(int d, int nx, int ntau, int nsys, bool mixed, bool cheb, bool ex, int nsm, size_t smem_sm, size_t smem_blk,
                int forms)
 {
-    OcPlan best = oc_choose(d, nx, ntau, nsys, mixed, cheb, ex, nsm, smem_sm, smem_blk, forms,
-                            [d](const OcPlan &p) { return kernel_regs(p, d); });
-    // The occupancy calculation has the last word.
-    if (best.ok && oc_max_blocks(best, d) * nsm < best.go * best.gt * nsys) best.ok = 0;
-    return best;
+    return oc_choose(
+        d, nx, ntau, nsys, mixed, cheb, ex, nsm, smem_sm, smem_blk, forms,
+        [d](const OcPlan &p) { return kernel_regs(p, d); },
+        [=](const OcPlan &p) { return oc_max_blocks(p, d) * nsm >= p.go * p.gt * nsys; });
 }
 
 cudaError_t oc_launch(const OcLaunch &L, const OcPlan &P, int d, cudaStream_t st)

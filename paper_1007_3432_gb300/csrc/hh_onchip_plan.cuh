@@ -34,17 +34,21 @@ inline bool cols_candidate(int d, long long P, int nx, int go, int so, int st, b
     return *threads <= col_max_threads(mixed ? 4 : 8, *K);
 }
 
-// The layout of least cost for nsys systems (ok = 0: none fits).  regs: registers per
-// thread of a layout's kernel.  forms as for oc_plan.
-template <typename Regs>
+// The layout of least cost for nsys systems (ok = 0: none fits).  regs_of: registers per
+// thread of a layout's kernel; fits: whether its blocks run on the chip at once, which
+// has the last word (when it refuses the best layout, the best one of another form or
+// number of blocks per SM is taken).  forms as for oc_plan.
+template <typename Regs, typename Fits>
 OcPlan oc_choose(int d, int nx, int ntau, int nsys, bool mixed, bool cheb, bool ex, int nsm, size_t smem_sm,
-                 size_t smem_blk, int forms, Regs &&regs_of)
+                 size_t smem_blk, int forms, Regs &&regs_of, Fits &&fits)
 {
-    OcPlan best = {};
+    constexpr int kMaxBlocks = 4, kForms = 3;
+    OcPlan found[kMaxBlocks][kForms] = {};      // best by blocks per SM and form
+    double costs[kMaxBlocks][kForms];
+    int order[kMaxBlocks][kForms], seen = 0;    // equal costs: the first one met
     const long long P = d == 3 ? (long long)nx * nx : 1;
-    double best_cost = 0.0;
     constexpr size_t kStatic = kOcStaticSmem;    // static and reserved shared memory per block
-    for (int m = 1; m <= 4; ++m) {
+    for (int m = 1; m <= kMaxBlocks; ++m) {
         const int G = (int)((long long)nsm * m / nsys) < kOcMaxTiles ? nsm * m / nsys : kOcMaxTiles;
         if (G < 1) continue;
         const int max_threads = kOcMaxThreads / m / 32 * 32;    // whole warps: the kernels sum by warps
@@ -88,7 +92,8 @@ OcPlan oc_choose(int d, int nx, int ntau, int nsys, bool mixed, bool cheb, bool 
                         if (form == 2) cost += 0.5 * m * C;
                     }
                     if (sm > kOcMaxSmem || sm + kStatic > smem_blk || (sm + kStatic) * m > smem_sm) continue;
-                    if (best.ok && cost >= best_cost) continue;
+                    OcPlan &best = found[m - 1][form];
+                    if (best.ok && cost >= costs[m - 1][form]) continue;
                     OcPlan p = {};
                     p.ok = 1;
                     p.go = go;
@@ -108,13 +113,28 @@ OcPlan oc_choose(int d, int nx, int ntau, int nsys, bool mixed, bool cheb, bool 
                     const int regs = (regs_of(p) + 7) / 8 * 8;
                     const int parts = (thr / 32 + 3) / 4;    // warps of a block per partition
                     if (regs <= 0 || 16384 / (regs * 32) / parts < m) continue;
-                    best_cost = cost;
+                    costs[m - 1][form] = cost;
+                    order[m - 1][form] = seen++;
                     best = p;
                 }
             }
         }
     }
-    return best;
+    for (;;) {
+        int bm = -1, bf = 0;
+        for (int m = 0; m < kMaxBlocks; ++m)
+            for (int f = 0; f < kForms; ++f) {
+                if (!found[m][f].ok) continue;
+                if (bm < 0 || costs[m][f] < costs[bm][bf] ||
+                    (costs[m][f] == costs[bm][bf] && order[m][f] < order[bm][bf])) {
+                    bm = m;
+                    bf = f;
+                }
+            }
+        if (bm < 0) return OcPlan{};
+        if (fits(found[bm][bf])) return found[bm][bf];
+        found[bm][bf].ok = 0;
+    }
 }
 
 }  // namespace hh

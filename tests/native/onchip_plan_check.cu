@@ -29,7 +29,8 @@ int main()
                                 const bool mixed = kind & 1, cheb = kind == 2, ex = kind >= 3;
                                 const hh::OcPlan p =
                                     hh::oc_choose(d, nx, ntau, nsys, mixed, cheb, ex, nsm, smem_sm, smem_blk, forms,
-                                                  [&](const hh::OcPlan &) { return regs; });
+                                                  [&](const hh::OcPlan &) { return regs; },
+                                                  [](const hh::OcPlan &) { return true; });
                                 if (!p.ok) continue;
                                 ++layouts;
 #define CHECK(cond, v) \
@@ -58,6 +59,18 @@ int main()
                                 CHECK((long long)p.go * p.gt * nsys <= m * nsm, m);
                             }
         }
+    // When the occupancy query refuses the best layout, the next one is taken: 32 x 64
+    // in FP64 is best in the column form, and fits in the tile form too.
+    for (bool refuse : {false, true}) {
+        const hh::OcPlan p = hh::oc_choose(1, 32, 64, 2, false, false, false, nsm, smem_sm, smem_blk, 1,
+                                           [](const hh::OcPlan &) { return 64; },
+                                           [=](const hh::OcPlan &q) { return !refuse || q.cols == 0; });
+        if (!p.ok || (p.cols == 0) != refuse) return fail("next layout", 1, 32, 64, 2, 64, p.cols);
+    }
+    const hh::OcPlan none = hh::oc_choose(1, 32, 64, 2, false, false, false, nsm, smem_sm, smem_blk, 1,
+                                          [](const hh::OcPlan &) { return 64; },
+                                          [](const hh::OcPlan &) { return false; });
+    if (none.ok) return fail("all refused", 1, 32, 64, 2, 64, none.cols);
     if (layouts < 10000) return fail("layouts", 0, 0, 0, 0, 0, layouts);
     std::printf("ok\n");
     return 0;
