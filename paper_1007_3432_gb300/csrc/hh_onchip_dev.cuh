@@ -114,18 +114,24 @@ __device__ __forceinline__ bool fetch(const unsigned char *buf, const int (&site
 // Sums of non-negative values in integers.  A shuffle tree of FP64 adds takes 80
 // clocks a level and 16 clocks of the SM's FP64 pipe per warp and level (1.4k
 // clocks for 16 warps); the integer warp reductions take 46 and none of it.
-// Each significand is shifted, rounding to nearest, to the largest exponent of
-// the warp and added as 27-bit parts: what a value loses is at most 2^-55 of
-// the largest, 32 times that for a warp, the bound of the FP64 tree (5 roundings
-// of 2^-53 of the sum) or less.
+// Each significand gets kGuardWarp more bits, is shifted, rounding to nearest, to
+// the largest exponent of the warp and added as 22-bit parts.  The largest value
+// is then at least 2^57 units and a shifted one loses at most half a unit: 31 of
+// them 31 2^-58, less than 2^-53 of the largest.  A block's warps are aligned and
+// added in the same way (15 2^-58), the total is rounded by 4 bits (2^-54) and to a
+// double (2^-53): less than 3 2^-53 of the sum, against the FP64 tree's 9
+// roundings of 2^-53 (5 levels of a warp, 4 of 16 warps).
+constexpr int kGuardWarp = 5;       // 32 values of 53 + 5 bits: 63 bits
+constexpr int kGuardSlots = 8;      // 5 values of 53 + 8 bits per lane: 64 bits
+constexpr int kNotFinite = 0x7fff;
+
 struct Significand {
-    int e;                  // biased FP64 exponent; 0x7ff: not finite
+    int e;                  // biased FP64 exponent; kNotFinite: infinity or NaN
     unsigned long long m;   // 53 bits
 };
 
-__device__ __forceinline__ Significand significand(double v)
+__host__ __device__ __forceinline__ Significand significand_bits(unsigned long long b)
 {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
     Significand p;
     p.e = (int)((b >> 52) & 0x7ffu);
     p.m = b & 0xfffffffffffffull;
@@ -133,12 +139,12 @@ __device__ __forceinline__ Significand significand(double v)
         p.m |= 1ull << 52;
     else
         p.e = 1;
+    if (p.e == 0x7ff) p.e = kNotFinite;
     return p;
 }
 
-__device__ __forceinline__ Significand significand(float v)
+__host__ __device__ __forceinline__ Significand significand_bits32(unsigned b)
 {
-    const unsigned b = __float_as_uint(v);
     int e = (int)((b >> 23) & 0xffu);
     unsigned m = b & 0x7fffffu;
     if (e)
@@ -146,56 +152,78 @@ __device__ __forceinline__ Significand significand(float v)
     else
         e = 1;
     Significand p;
-    p.e = e == 255 ? 0x7ff : e + (1023 - 127);
+    p.e = e == 255 ? kNotFinite : e + (1023 - 127);
     p.m = (unsigned long long)m << 29;
     return p;
 }
 
-// v / 2^d, rounded to nearest (d >= 0, v < 2^62).
-__device__ __forceinline__ unsigned long long shift_round(unsigned long long v, int d)
+__device__ __forceinline__ Significand significand(double v)
+{
+    return significand_bits((unsigned long long)__double_as_longlong(v));
+}
+
+__device__ __forceinline__ Significand significand(float v)
+{
+    return significand_bits32(__float_as_uint(v));
+}
+
+// v / 2^d, rounded to nearest (d >= 0, v < 2^63; 0 from d = 63 on).
+__host__ __device__ __forceinline__ unsigned long long shift_round(unsigned long long v, int d)
 {
     return d > 62 ? 0ull : (v + ((1ull << d) >> 1)) >> d;
 }
 
-// A sum s 2^(e - 1076); e = 0x7ff: not finite.
+// A sum s 2^(e - 1075 - kGuardWarp), s < 2^63; e >= kNotFinite: not finite.
 struct ISum {
     unsigned long long s;
     int e;
 };
 
-// Sum over the warp, the same in every lane: s < 2^59.
+// The total s2 2^44 + s1 2^22 + s0 of a warp's parts (s1, s0 < 2^27), divided by
+// 2^shift and rounded to nearest.
+__host__ __device__ __forceinline__ unsigned long long isum_join(unsigned long long s2, unsigned long long s1,
+                                                                 unsigned long long s0, int shift)
+{
+    return (s2 << (44 - shift)) + (((s1 << 22) + s0 + ((1ull << shift) >> 1)) >> shift);
+}
+
+// Sum over the warp of one aligned term per lane, divided by 2^shift.
+__device__ __forceinline__ unsigned long long warp_join(unsigned long long x, int shift)
+{
+    const unsigned s2 = __reduce_add_sync(0xffffffffu, (unsigned)(x >> 44));
+    const unsigned s1 = __reduce_add_sync(0xffffffffu, (unsigned)(x >> 22) & 0x3fffffu);
+    const unsigned s0 = __reduce_add_sync(0xffffffffu, (unsigned)x & 0x3fffffu);
+    return isum_join(s2, s1, s0, shift);
+}
+
+// Sum over the warp, the same in every lane.
 template <typename T>
 __device__ __forceinline__ ISum warp_isum(T v)
 {
     const Significand p = significand(v);
     ISum r;
     r.e = (int)__reduce_max_sync(0xffffffffu, (unsigned)p.e);
-    const unsigned long long x = shift_round(p.m << 1, r.e - p.e);
-    const unsigned long long hi = __reduce_add_sync(0xffffffffu, (unsigned)(x >> 27));
-    const unsigned long long lo = __reduce_add_sync(0xffffffffu, (unsigned)x & 0x7ffffffu);
-    r.s = (hi << 27) + lo;
+    r.s = warp_join(shift_round(p.m << kGuardWarp, r.e - p.e), 0);
     return r;
 }
 
-__device__ __forceinline__ double isum_value(const ISum &a)
+// The value of s 2^(e - 1075 - guard).
+__device__ __forceinline__ double isum_value(const ISum &a, int guard = kGuardWarp)
 {
-    if (a.e == 0x7ff) return __longlong_as_double((long long)kSigNaN);
+    if (a.e >= kNotFinite) return __longlong_as_double((long long)kSigNaN);
     const double v = __ull2double_rn(a.s);
-    const int e = (int)((unsigned long long)__double_as_longlong(v) >> 52) + a.e - 1076;
-    if (a.s == 0ull || e < 1 || e > 2046) return scalbn(v, a.e - 1076);
-    return __longlong_as_double(__double_as_longlong(v) + ((long long)(a.e - 1076) << 52));
+    const int k = a.e - 1075 - guard, e = (int)((unsigned long long)__double_as_longlong(v) >> 52) + k;
+    if (a.s == 0ull || e < 1 || e > 2046) return scalbn(v, k);
+    return __longlong_as_double(__double_as_longlong(v) + ((long long)k << 52));
 }
 
-// Sum over the warp of one partial sum per lane (s < 2^59; 16 lanes' worth at most are not zero).
+// Sum over the warp of one partial sum per lane (at most 16 of them not zero).
 __device__ __forceinline__ ISum warp_isum_parts(const ISum &a)
 {
     ISum r;
     r.e = (int)__reduce_max_sync(0xffffffffu, (unsigned)a.e);
-    const unsigned long long x = shift_round(a.s, r.e - a.e);
-    const unsigned long long s2 = __reduce_add_sync(0xffffffffu, (unsigned)(x >> 44));
-    const unsigned long long s1 = __reduce_add_sync(0xffffffffu, (unsigned)(x >> 22) & 0x3fffffu);
-    const unsigned long long s0 = __reduce_add_sync(0xffffffffu, (unsigned)x & 0x3fffffu);
-    r.s = (s2 << 44) + (s1 << 22) + s0;
+    r.s = warp_join(shift_round(a.s, r.e - a.e), 4);
+    r.e += 4;
     return r;
 }
 
@@ -247,7 +275,7 @@ __device__ __forceinline__ bool sum_slots(const Raw16 *slot, int n, uint32_t seq
             }
             acc.e = (int)__reduce_max_sync(0xffffffffu, (unsigned)em);
 #pragma unroll
-            for (int u = 0; u < U; ++u) acc.s += shift_round(p[u].m << 1, acc.e - p[u].e);
+            for (int u = 0; u < U; ++u) acc.s += shift_round(p[u].m << kGuardSlots, acc.e - p[u].e);
         } else {
             const double a01 = __longlong_as_double((long long)a[0].v) + __longlong_as_double((long long)a[1].v);
             const double a23 = __longlong_as_double((long long)a[2].v) + __longlong_as_double((long long)a[3].v);
@@ -256,11 +284,9 @@ __device__ __forceinline__ bool sum_slots(const Raw16 *slot, int n, uint32_t seq
     }
     ok = __all_sync(0xffffffffu, ok);
     if (NONNEG && n <= 32 * U) {
-        const unsigned long long s2 = __reduce_add_sync(0xffffffffu, (unsigned)(acc.s >> 44));
-        const unsigned long long s1 = __reduce_add_sync(0xffffffffu, (unsigned)(acc.s >> 22) & 0x3fffffu);
-        const unsigned long long s0 = __reduce_add_sync(0xffffffffu, (unsigned)acc.s & 0x3fffffu);
-        acc.s = (s2 << 44) + (s1 << 22) + s0;
-        sum = isum_value(acc);
+        // 160 values of 61 bits: 159 2^-61 lost in the alignment, 2^-53 and less in the roundings.
+        acc.s = warp_join(acc.s, 5);
+        sum = isum_value(acc, kGuardSlots - 5);
     } else {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);

@@ -148,3 +148,32 @@ def test_plain_c_program_links_against_the_library(tmp_path):
     links against the built library; tests/test_gpu_c_consumer.py runs it."""
     exe, _ = build_c_consumer(tmp_path)
     assert os.path.exists(exe)
+
+
+def onchip_math_check(tmp_path, *args):
+    import shutil
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    exe = str(tmp_path / "onchip_math_check")
+    subprocess.check_call([nvcc, "-O2", "-std=c++17", "-gencode", "arch=compute_103a,code=sm_103a",
+                           "-I", os.path.join(ROOT, "include"),
+                           os.path.join(ROOT, "tests", "native", "onchip_math_check.cu"), "-o", exe])
+    out = subprocess.run([exe, *args], capture_output=True, text=True)
+    assert out.returncode == 0 and out.stdout.strip().endswith("ok"), out.stdout + out.stderr
+    return out.stdout
+
+
+def test_onchip_integer_sums(tmp_path):
+    """The integer sums of the on-chip engine, emulated on the host, stay
+    within their stated error bounds (one large value among many small ones
+    that all round the same way included)."""
+    onchip_math_check(tmp_path)
+
+
+@pytest.mark.gpu
+def test_onchip_integer_sums_and_quotients_on_the_gpu(tmp_path):
+    """The device functions: sums bit for bit the emulated ones, quotients
+    against the division over 640,000 draws."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    onchip_math_check(tmp_path, "gpu")
