@@ -117,10 +117,10 @@ __device__ __forceinline__ bool fetch(const unsigned char *buf, const int (&site
 // Each significand gets kGuardWarp more bits, is shifted, rounding to nearest, to
 // the largest exponent of the warp and added as 22-bit parts.  The largest value
 // is then at least 2^57 units and a shifted one loses at most half a unit: 31 of
-// them 31 2^-58, less than 2^-53 of the largest.  A block's warps are aligned and
-// added in the same way (15 2^-58), the total is rounded by 4 bits (2^-54) and to a
-// double (2^-53): less than 3 2^-53 of the sum, against the FP64 tree's 9
-// roundings of 2^-53 (5 levels of a warp, 4 of 16 warps).
+// them 31 2^-58, less than 2^-53 of the largest.  A block's warps are normalised to 55
+// bits and added in two parts (15 2^-55 at most), and the total is rounded to a double
+// (2^-53): less than 6 2^-53 of the sum, against the FP64 tree's 9 roundings of 2^-53
+// (5 levels of a warp, 4 of 16 warps).
 constexpr int kGuardWarp = 5;       // 32 values of 53 + 5 bits: 63 bits
 constexpr int kGuardSlots = 8;      // 5 values of 53 + 8 bits per lane: 64 bits
 constexpr int kNotFinite = 0x7fff;
@@ -167,7 +167,7 @@ __device__ __forceinline__ Significand significand(float v)
     return significand_bits32(__float_as_uint(v));
 }
 
-// v / 2^d, rounded to nearest (d >= 0, v < 2^63; 0 from d = 63 on).
+// v / 2^d, rounded to nearest (d >= 0, v < 2^62).
 __host__ __device__ __forceinline__ unsigned long long shift_round(unsigned long long v, int d)
 {
     return d > 62 ? 0ull : (v + ((1ull << d) >> 1)) >> d;
@@ -217,13 +217,45 @@ __device__ __forceinline__ double isum_value(const ISum &a, int guard = kGuardWa
     return __longlong_as_double(__double_as_longlong(v) + ((long long)k << 52));
 }
 
+// A partial sum as 64 bits with the highest one set, and the exponent of that bit
+// (in the units of e): s = 0 has exponent 0.
+struct Normal {
+    unsigned long long v;
+    int e;
+};
+
+__host__ __device__ __forceinline__ Normal isum_normal(const ISum &a)
+{
+#ifdef __CUDA_ARCH__
+    const int z = __clzll((long long)a.s);
+#else
+    const int z = a.s ? __builtin_clzll(a.s) : 64;
+#endif
+    Normal r;
+    r.v = z < 64 ? a.s << z : 0ull;
+    r.e = a.e >= kNotFinite ? 2 * kNotFinite : z < 64 ? a.e + 64 - z : 0;
+    return r;
+}
+
+// Its 55 bits (56 when rounding carries) aligned to the largest exponent.
+__host__ __device__ __forceinline__ unsigned long long normal_term(const Normal &a, int emax)
+{
+    const int d = 8 + emax - a.e;
+    const unsigned long long w = d > 63 ? 0ull : a.v >> d;
+    return (w >> 1) + (w & 1ull);
+}
+
 // Sum over the warp of one partial sum per lane (at most 16 of them not zero).
 __device__ __forceinline__ ISum warp_isum_parts(const ISum &a)
 {
+    const Normal n = isum_normal(a);
     ISum r;
-    r.e = (int)__reduce_max_sync(0xffffffffu, (unsigned)a.e);
-    r.s = warp_join(shift_round(a.s, r.e - a.e), 4);
-    r.e += 4;
+    r.e = (int)__reduce_max_sync(0xffffffffu, (unsigned)n.e);
+    const unsigned long long x = normal_term(n, r.e);
+    const unsigned hi = __reduce_add_sync(0xffffffffu, (unsigned)(x >> 28));
+    const unsigned lo = __reduce_add_sync(0xffffffffu, (unsigned)x & 0xfffffffu);
+    r.s = ((unsigned long long)hi << 28) + lo;
+    r.e -= 55;
     return r;
 }
 
