@@ -218,7 +218,9 @@ int hh_apply_multi(hh_ctx *ctx, int op, const void *x, void *y, int n_vec, int d
  * P(Q) of Sec. 4.2, applied as n real quadratic factors (2n applications of
  * Q per step); info->iterations then counts preconditioned steps.
  * b, x: device pointers to n_rhs * N doubles.  info may be NULL (then the call
- * does not synchronise).  Returns HH_ENOCONV if a right-hand side missed
+ * does not synchronise, and may be captured into a CUDA graph: a captured solve
+ * brings its own tables and may be replayed after other solves of the context,
+ * on its stream).  Returns HH_ENOCONV if a right-hand side missed
  * cg_tol within cg_maxit (x then holds the last iterate), HH_ETIMEOUT if a
  * bounded device-side wait ran out, HH_ENUMERIC on NaN/Inf. */
 int hh_solve(hh_ctx *ctx, const double *b, double *x, int n_rhs, hh_solve_info *info);

@@ -31,12 +31,38 @@ struct EngStats {
     double max_relres;
 };
 
-// New solves: states MODE_NEW, empty signal slots for 'parts' tile partials,
-// iteration counter 0; the on-chip engine's phase numbers (seq, may be null)
-// go on from where the last launch ended.
-__global__ void k_engine_reset(EngState *s0, EngState *s1, int nsys, unsigned long long *sig, int parts,
+// The systems of a solve, by value in the parameters of the kernel that starts it.
+template <int CAP>
+struct SysTable {
+    EngSystem sys[CAP];
+};
+constexpr int kSmallTable = 4, kLargeTable = 64;     // n_pf <= 64
+
+// Starts a solve: its system and tile tables, states MODE_NEW, empty signal slots for
+// 'parts' tile partials, iteration counter 0; the on-chip engine's phase numbers
+// (seq, may be null) go on from where the last launch ended.  The tables come with
+// every solve, so that a captured one finds its own when it is replayed, whatever
+// the context has solved since.
+template <int CAP>
+__global__ void k_engine_reset(const __grid_constant__ SysTable<CAP> tab, EngSystem *sys, EngTile *tiles, int chunk,
+                               EngState *s0, EngState *s1, int nsys, unsigned long long *sig, int parts,
                                EngCtl *ctl, long long timeout_ns, int drop_sig, unsigned long long *seq)
 {
+    static_assert(sizeof(EngSystem) % 8 == 0, "copied in words");
+    constexpr int W = sizeof(EngSystem) / 8;
+    const unsigned long long *const src = (const unsigned long long *)&tab;
+    for (int j = threadIdx.x; j < nsys * W; j += blockDim.x) ((unsigned long long *)sys)[j] = src[j];
+    // Tiles of 'chunk' sites of one system after the other; their number is the
+    // same for all (equal lattices), and so is the order of their partial sums.
+    const int per = tab.sys[0].ntiles, N = tab.sys[0].g.N;
+    for (int j = threadIdx.x; j < nsys * per; j += blockDim.x) {
+        EngTile T;
+        T.sys = j / per;
+        T.begin = (j - T.sys * per) * chunk;
+        T.end = N - T.begin > chunk ? T.begin + chunk : N;
+        T.part = j;
+        tiles[j] = T;
+    }
     for (int s = threadIdx.x; s < nsys; s += blockDim.x) {
         EngState z;
         memset(&z, 0, sizeof(z));
@@ -111,14 +137,14 @@ __global__ void k_zero_stats(EngStats *stats)
     if (threadIdx.x == 0) memset(stats, 0, sizeof(EngStats));
 }
 
-// Plan of one engine launch: the system table and tiles in device memory.
+// Plan of one engine launch.
 struct Plan {
-    int nsys = 0, ntiles = 0, grid = 0, homogeneous = 0;
+    int nsys = 0, ntiles = 0, chunk = 0, grid = 0, homogeneous = 0;
     int precision = -1;
     int x0 = 0;                  // systems start from the x passed in
     const double *b = nullptr;
     double *x = nullptr;
-    EngSystem sys[64];           // host copy of the device system table (n_pf <= 64)
+    EngSystem sys[kLargeTable];  // the systems; each solve writes them to the device
     OcPlan oc;                   // layout of the on-chip engine (ok = 0: the grid engine)
 };
 
@@ -318,12 +344,9 @@ int make_plan(hh_ctx *c, const double *b, double *x, int n_rhs)
     // t, x, links, p' in FP32 (mixed).
     const long long site_bytes = mixed ? 24 : (c->prm.cheb_degree > 0 ? 72 : 56);
     const int pf = engine_prefetch(site_bytes * (long long)c->N * n_rhs, c->lat.d);
-    std::vector<EngSystem> sys(n_rhs);
-    std::vector<EngTile> tiles;
-    tiles.reserve(ntiles);
-    const int chunk = tl.chunk;
+    const int tps = tl.tiles;
     for (int a = 0; a < n_rhs; ++a) {
-        EngSystem &Y = sys[a];
+        EngSystem &Y = P.sys[a];
         memset(&Y, 0, sizeof(Y));
         Y.g = c->geo;
         Y.h = c->prm.t * c->prm.dtau;
@@ -341,16 +364,8 @@ int make_plan(hh_ctx *c, const double *b, double *x, int n_rhs)
         Y.p32b = c->p32b + off;
         Y.t32 = c->t32 + off;
         Y.x32 = c->x32 + off;
-        Y.tile0 = (int)tiles.size();
-        for (int s0 = 0; s0 < c->N; s0 += chunk) {
-            EngTile T;
-            T.sys = a;
-            T.begin = s0;
-            T.end = s0 + chunk < c->N ? s0 + chunk : c->N;
-            T.part = (int)tiles.size();
-            tiles.push_back(T);
-        }
-        Y.ntiles = (int)tiles.size() - Y.tile0;
+        Y.tile0 = a * tps;
+        Y.ntiles = tps;
         Y.part0 = Y.tile0;
         Y.owner = overlap ? a % grid : Y.tile0 % grid;
         Y.precision = mixed ? PREC_MIXED : PREC_FP64;
@@ -369,16 +384,10 @@ int make_plan(hh_ctx *c, const double *b, double *x, int n_rhs)
         Y.z = c->z ? c->z + off : nullptr;
         Y.u = c->u ? c->u + off : nullptr;
     }
-    ntiles = (int)tiles.size();
-    // Pageable sources: the copies have consumed the host buffers on return.
-    HH_TRY(cudaMemcpyAsync(c->d_sys, sys.data(), sizeof(EngSystem) * n_rhs, cudaMemcpyHostToDevice,
-                           c->stream));
-    for (int a = 0; a < n_rhs; ++a) P.sys[a] = sys[a];
     P.x0 = 0;
-    HH_TRY(cudaMemcpyAsync(c->d_tiles, tiles.data(), sizeof(EngTile) * ntiles,
-                           cudaMemcpyHostToDevice, c->stream));
     P.nsys = n_rhs;
     P.ntiles = ntiles;
+    P.chunk = tl.chunk;
     P.grid = grid;
     P.homogeneous = overlap ? 1 : 0;
     P.b = b;
@@ -389,16 +398,25 @@ int make_plan(hh_ctx *c, const double *b, double *x, int n_rhs)
 }
 
 // Whether the plan's systems start from the x passed in (an initial guess) or
-// from x = 0; re-uploads the system table when that changes.
-int set_guess(hh_ctx *c, int x0)
+// from x = 0.
+void set_guess(hh_ctx *c, int x0)
 {
     Plan &P = c->plan;
-    if (P.x0 == x0) return HH_OK;
+    if (P.x0 == x0) return;
     for (int a = 0; a < P.nsys; ++a) P.sys[a].x0_given = x0;
-    // Pageable source: the copy has consumed it on return.
-    HH_TRY(cudaMemcpyAsync(c->d_sys, P.sys, sizeof(EngSystem) * P.nsys, cudaMemcpyHostToDevice, c->stream));
     P.x0 = x0;
-    return HH_OK;
+}
+
+template <int CAP>
+cudaError_t launch_reset(hh_ctx *c)
+{
+    const Plan &P = c->plan;
+    SysTable<CAP> tab;
+    memcpy(tab.sys, P.sys, sizeof(EngSystem) * P.nsys);
+    k_engine_reset<CAP><<<1, 256, 0, c->stream>>>(tab, c->d_sys, c->d_tiles, P.chunk, c->d_state[0], c->d_state[1],
+                                                  P.nsys, c->d_sig, c->max_tiles, c->d_ctl, c->timeout_ns,
+                                                  engine_drop_signal(), c->d_seq);
+    return cudaGetLastError();
 }
 
 // The force from the solutions in xsol (n_rhs right-hand sides): pi -= eps F
@@ -422,10 +440,7 @@ int run_engine(hh_ctx *c)
 {
     TraceRange tr("hh engine solve");
     const Plan &P = c->plan;
-    k_engine_reset<<<1, 256, 0, c->stream>>>(c->d_state[0], c->d_state[1], P.nsys, c->d_sig,
-                                             c->max_tiles, c->d_ctl, c->timeout_ns, engine_drop_signal(),
-                                             c->d_seq);
-    HH_TRY(cudaGetLastError());
+    HH_TRY(P.nsys <= kSmallTable ? launch_reset<kSmallTable>(c) : launch_reset<kLargeTable>(c));
     bool rec = c->profile && c->ev_used + 2 <= c->ev_cap;
     if (rec) HH_TRY(cudaEventRecord(c->ev[c->ev_used], c->stream));
     // A mixed system that ends in FP64 steps leaves the on-chip engine for the
@@ -976,8 +991,7 @@ static int solve_from(hh_ctx *c, const double *b, double *x, int n_rhs, int x0, 
     if (rc) return rc;
     rc = make_plan(c, b, x, n_rhs);
     if (rc) return rc;
-    rc = set_guess(c, x0);
-    if (rc) return rc;
+    set_guess(c, x0);
     k_zero_stats<<<1, 32, 0, c->stream>>>(c->d_stats);
     HH_TRY(cudaGetLastError());
     c->n_launch += 1;
@@ -1008,8 +1022,7 @@ int hh_force(hh_ctx *c, const double *chi, int n_rhs, double *F, hh_solve_info *
     if (rc) return rc;
     rc = make_plan(c, chi, c->xsol, n_rhs);
     if (rc) return rc;
-    rc = set_guess(c, 0);
-    if (rc) return rc;
+    set_guess(c, 0);
     k_zero_stats<<<1, 32, 0, c->stream>>>(c->d_stats);
     HH_TRY(cudaGetLastError());
     c->n_launch += 1;
@@ -1034,8 +1047,7 @@ int hh_action(hh_ctx *c, const double *chi, int n_rhs, double *S, hh_solve_info 
     if (rc) return rc;
     rc = make_plan(c, chi, c->xsol, n_rhs);
     if (rc) return rc;
-    rc = set_guess(c, 0);
-    if (rc) return rc;
+    set_guess(c, 0);
     k_zero_stats<<<1, 32, 0, c->stream>>>(c->d_stats);
     HH_TRY(cudaGetLastError());
     c->n_launch += 1;
@@ -1135,8 +1147,7 @@ int leapfrog_enqueue(hh_ctx *c, double *pi, const double *chi, int n_rhs, int n_
             HH_TRY(cudaMemcpyAsync(c->xprev, c->xsol, sizeof(double) * (size_t)nx, cudaMemcpyDeviceToDevice,
                                    c->stream));
         }
-        rc = set_guess(c, (chrono != 0 && j >= 1) ? 1 : 0);
-        if (rc) return rc;
+        set_guess(c, (chrono != 0 && j >= 1) ? 1 : 0);
         rc = run_engine(c);
         if (rc) return rc;
         if (j == 0 && h0)

@@ -208,3 +208,45 @@ def test_onchip_solve_replays_from_a_graph(hh, monkeypatch, precision):
                 x.zero_()
                 ctx.solve(b, x, 1)
                 assert torch.equal(x, ref)
+
+
+@pytest.mark.parametrize("onchip", [0, 1])
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_captured_solve_replays_after_other_solves(hh, monkeypatch, onchip, precision):
+    """A captured solve brings its own system and tile tables: replays after
+    solves of other right-hand sides (more of them, from a guess) give its own
+    bits; so do those solves after the replay."""
+    monkeypatch.setenv("HH_ENGINE_ONCHIP", str(onchip))
+    d, nx, ntau = 1, 48, 24
+    n = nx * ntau
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        sigma = dev(workloads.sigma_field(n, seed=2201))
+        b = dev(np.stack([workloads.source(n, seed=2200, rhs=a) for a in range(6)]))
+        two, five = torch.zeros_like(b[:2]), torch.zeros_like(b[1:])
+        for ref, rhs in ((two, b[:2]), (five, b[1:])):
+            with hh.Context(d, nx, ntau, precision=precision, n_pf=5) as ctx:
+                ctx.set_field(sigma)
+                ctx.solve(rhs, ref, ref.shape[0])
+        with hh.Context(d, nx, ntau, precision=precision, n_pf=5) as ctx:
+            ctx.set_field(sigma)
+            xa, xb = torch.zeros_like(two), torch.zeros_like(five)
+            ctx.solve(b[:2], xa, 2)
+            stream.synchronize()
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=stream):
+                ctx.solve(b[:2], xa, 2, info=False)
+            for guess in (False, True):
+                xa.zero_()
+                g.replay()
+                stream.synchronize()
+                assert torch.equal(xa, two)
+                xb.zero_()
+                ctx.solve(b[1:], xb, 5)
+                assert torch.equal(xb, five)
+                xa.zero_()
+                g.replay()
+                stream.synchronize()
+                assert torch.equal(xa, two)
+                ctx.solve(b[1:], xb, 5, guess=guess)    # the same plan as before the replay
+                assert torch.equal(xb, five)
