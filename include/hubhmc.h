@@ -164,7 +164,10 @@ void hh_default_params(hh_params *p);
 
 /* Create a context for one lattice and one Markov chain.  Allocates sigma,
  * the links (FP64 and FP32), the HMC fields and the CG workspace on the
- * current device.  stream: a cudaStream_t (NULL = legacy default stream).
+ * current device; for lattices whose CG vectors can stay on the chip also that
+ * engine's exchange buffers (32 bytes per site and right-hand side in HH_FP64, 16
+ * in HH_MIXED, and 152 KB per right-hand side; without room for them the engine
+ * that streams the vectors solves every system).  Solves allocate nothing.  stream: a cudaStream_t (NULL = legacy default stream).
  * sigma starts at zero.  Errors: HH_EINVAL (d not 1 or 3, nx < 2, ntau < 2,
  * N >= 2^31, n_pf < 1, unknown precision), HH_ENOMEM, HH_ECUDA. */
 int hh_create(hh_ctx **out, const hh_lattice *lat, const hh_params *p, void *cuda_stream);

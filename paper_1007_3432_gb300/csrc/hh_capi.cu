@@ -177,16 +177,13 @@ struct hh_ctx {
     EngStats *d_stats;
     int max_tiles;
     Plan plan;
-    // On-chip engine: one block of device memory, allocated by the first plan that
-    // uses it: partial-sum packets, phase numbers, packets of two vectors per
-    // system (for oc_cap systems), and the number of systems the packets were last
-    // used for.
+    // On-chip engine: one block of device memory for oc_cap systems (0: no lattice of this
+    // size fits): partial-sum packets, phase numbers, packets of two vectors per system;
+    // and the number of systems the packets were last used for.
     unsigned char *d_pkt;
     ulonglong2 *d_slots;
     unsigned long long *d_seq;
     int oc_cap, oc_last;
-    void *oc_old[65];       // blocks that a larger one has replaced: a captured solve may be
-    int n_oc_old;           // replayed on them, so they live as long as the context
     int oc_forms;           // on-chip engine: 0 not used, 1 by rule, 2 tile form, 3 column form only
     bool oc_known[65];      // layouts by number of systems (n_pf <= 64), once computed
     OcPlan oc_plans[65];
@@ -255,7 +252,6 @@ void free_ctx(hh_ctx *c)
         if (p) cudaFree(p);
     if (c->L16) cudaFree(c->L16);
     if (c->d_slots) cudaFree(c->d_slots);    // d_seq and d_pkt lie behind it
-    for (int i = 0; i < c->n_oc_old; ++i) cudaFree(c->oc_old[i]);
     if (c->ev) {
         for (int i = 0; i < c->ev_cap; ++i)
             if (c->ev[i]) cudaEventDestroy(c->ev[i]);
@@ -281,12 +277,33 @@ int oc_allowed(const hh_ctx *c)
     return e ? atoi(e) : 1;
 }
 
-// Layout of the on-chip engine for n_rhs systems, with its device memory; ok = 0:
-// the grid engine solves them.
+// The on-chip engine's device memory, allocated with the context so that solves do not
+// allocate.  Without room for it (false) the grid engine solves everything.
+bool oc_alloc(hh_ctx *c)
+{
+    if (c->oc_forms <= 0) return true;
+    const long long fit = oc_most_systems(c->N, c->prm.precision != HH_FP64, c->nsm, (size_t)c->smem_sm);
+    const int most = fit < c->cap_rhs ? (int)fit : c->cap_rhs;
+    if (most == 0) return true;
+    const size_t sb = sizeof(ulonglong2) * 2 * kOcReplicas * kOcMaxTiles * (size_t)most;
+    const size_t bytes = sb + 256 + oc_packets(c, most);
+    unsigned char *blk = nullptr;
+    if (cudaMalloc((void **)&blk, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    c->d_slots = (ulonglong2 *)blk;
+    c->d_seq = (unsigned long long *)(blk + sb);
+    c->d_pkt = blk + sb + 256;
+    c->oc_cap = most;
+    return cudaMemsetAsync(blk, 0, bytes, c->stream) == cudaSuccess;
+}
+
+// Layout of the on-chip engine for n_rhs systems; ok = 0: the grid engine solves them.
 OcPlan ctx_oc_plan(hh_ctx *c, int n_rhs)
 {
     OcPlan none = {};
-    if (c->oc_forms <= 0) return none;
+    if (n_rhs > c->oc_cap) return none;
     if (!c->oc_known[n_rhs]) {
         const bool mixed = c->prm.precision != HH_FP64;
         c->oc_plans[n_rhs] = oc_plan(c->lat.d, c->lat.nx, c->lat.ntau, n_rhs, mixed, c->prm.cheb_degree > 0,
@@ -296,23 +313,6 @@ OcPlan ctx_oc_plan(hh_ctx *c, int n_rhs)
     }
     const OcPlan &p = c->oc_plans[n_rhs];
     if (!p.ok) return none;
-    if (n_rhs > c->oc_cap) {
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return none;
-        const size_t sb = sizeof(ulonglong2) * 2 * kOcReplicas * kOcMaxTiles * (size_t)n_rhs;
-        unsigned char *blk = nullptr;
-        if (cudaMalloc((void **)&blk, sb + 256 + oc_packets(c, n_rhs)) != cudaSuccess) {
-            cudaGetLastError();
-            return none;
-        }
-        if (c->d_slots) c->oc_old[c->n_oc_old++] = c->d_slots;
-        c->d_slots = (ulonglong2 *)blk;
-        c->d_seq = (unsigned long long *)(blk + sb);
-        c->d_pkt = blk + sb + 256;
-        c->oc_cap = n_rhs;
-        c->oc_last = 0;
-        if (cudaMemsetAsync(blk, 0, sb + 256, c->stream) != cudaSuccess) return none;
-    }
     // Other tiles publish other sites: forget the packets of the last layout.
     if (c->oc_last != n_rhs) {
         if (cudaMemsetAsync(c->d_pkt, 0, oc_packets(c, c->oc_cap), c->stream) != cudaSuccess) return none;
@@ -753,6 +753,7 @@ int hh_create(hh_ctx **out, const hh_lattice *lat, const hh_params *p, void *cud
         e = dalloc(&c->L16, n);
     }
     c->oc_forms = oc_allowed(c);
+    if (e == cudaSuccess && !oc_alloc(c)) c->oc_forms = 0;
     if (e == cudaSuccess) e = launch_links(c->geo, p->A, c->sigma, c->L64, c->L32, c->stream);
     if (e == cudaSuccess) e = links16_after(c);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);

@@ -77,6 +77,13 @@ inline size_t oc_packet_bytes(bool mixed) { return mixed ? 8 : 16; }
 constexpr int kOcMaxTiles = 608;
 constexpr int kOcReplicas = 8;
 
+// Systems of N sites that can lie on the chip at most: the tile form keeps at least four
+// vectors (links, p, t, r) in shared memory, the column form's registers hold fewer sites.
+inline long long oc_most_systems(long long N, bool mixed, int nsm, size_t smem_sm)
+{
+    return (long long)nsm * (long long)(smem_sm / (4 * (mixed ? 4 : 8))) / N;
+}
+
 // Layout for nsys systems, on nsm SMs with smem_sm bytes of shared memory per
 // SM and smem_blk at most per block.  forms: 1 the faster form, 2 the tile form,
 // 3 the column form only.

@@ -57,6 +57,9 @@ int main()
                                 if (rm < m) m = rm;
                                 CHECK(p.smem + 1024 <= smem_blk, p.smem);
                                 CHECK((long long)p.go * p.gt * nsys <= m * nsm, m);
+                                // The exchange buffers are allocated for these many.
+                                const long long N = (long long)P * nx * ntau;
+                                CHECK(nsys <= hh::oc_most_systems(N, mixed, nsm, smem_sm), N);
                             }
         }
     // When the occupancy query refuses the best layout, the next one is taken: 32 x 64

@@ -213,7 +213,8 @@ def test_onchip_solve_replays_from_a_graph(hh, monkeypatch, precision):
 @pytest.mark.parametrize("onchip", [0, 1])
 @pytest.mark.parametrize("precision", ["fp64", "mixed"])
 def test_captured_solve_replays_after_other_solves(hh, monkeypatch, onchip, precision):
-    """A captured solve brings its own system and tile tables: replays after
+    """A captured solve brings its own system and tile tables and, also as the
+    context's first solve, runs in the same engine as others: replays after
     solves of other right-hand sides (more of them, from a guess) give its own
     bits; so do those solves after the replay."""
     monkeypatch.setenv("HH_ENGINE_ONCHIP", str(onchip))
@@ -231,7 +232,6 @@ def test_captured_solve_replays_after_other_solves(hh, monkeypatch, onchip, prec
         with hh.Context(d, nx, ntau, precision=precision, n_pf=5) as ctx:
             ctx.set_field(sigma)
             xa, xb = torch.zeros_like(two), torch.zeros_like(five)
-            ctx.solve(b[:2], xa, 2)
             stream.synchronize()
             g = torch.cuda.CUDAGraph()
             with torch.cuda.graph(g, stream=stream):
@@ -250,3 +250,30 @@ def test_captured_solve_replays_after_other_solves(hh, monkeypatch, onchip, prec
                 assert torch.equal(xa, two)
                 ctx.solve(b[1:], xb, 5, guess=guess)    # the same plan as before the replay
                 assert torch.equal(xb, five)
+
+
+def test_first_solves_allocate_nothing(hh, monkeypatch):
+    """Solves take no device memory, the first one and larger ones included:
+    another stream's capture may be going on (an allocation would end it)."""
+    monkeypatch.setenv("HH_ENGINE_ONCHIP", "1")
+    d, nx, ntau = 1, 64, 16
+    n = nx * ntau
+    b = dev(np.stack([workloads.source(n, seed=2300, rhs=a) for a in range(4)]))
+    x = torch.zeros_like(b)
+    y = torch.zeros(8, device="cuda")
+    own, side = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with hh.Context(d, nx, ntau, stream=own) as ctx:
+        ctx.set_field(dev(workloads.sigma_field(n, seed=2301)))
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=side):        # global capture mode
+            y += 1.0
+            for k in (1, 3, 4):
+                ctx.solve(b, x, k, info=False)
+        torch.cuda.synchronize()
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.all(y == 1.0)
+        rc, info = ctx.solve(b, x, 4)
+        assert rc == 0 and info["converged"] == 1
