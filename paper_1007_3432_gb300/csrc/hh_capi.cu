@@ -78,7 +78,7 @@ __global__ void k_engine_reset(const __grid_constant__ SysTable<CAP> tab, EngSys
         ctl->k_end = 0;
         ctl->timeout_ns = timeout_ns;
         ctl->drop_sig = drop_sig;
-        if (seq) seq[0] = seq[1] + 1;
+        if (seq) seq[0] = oc_first_phase(seq[1]);
     }
 }
 

@@ -77,6 +77,16 @@ inline size_t oc_packet_bytes(bool mixed) { return mixed ? 8 : 16; }
 constexpr int kOcMaxTiles = 608;
 constexpr int kOcReplicas = 8;
 
+// First phase number of a launch after 'last', the last of the launches before it.
+// Packets compare its low 32 bits and cleared ones carry 0, so a launch that could
+// reach a multiple of 2^32 (2^28 phases are minutes of one solve) starts behind it.
+__host__ __device__ inline unsigned long long oc_first_phase(unsigned long long last)
+{
+    const unsigned long long first = last + 1, low = first & 0xffffffffull;
+    if (low == 0) return first + 1;
+    return low > 0xf0000000ull ? (((first >> 32) + 1) << 32) + 1 : first;
+}
+
 // Systems of N sites that can lie on the chip at most: the tile form keeps at least four
 // vectors (links, p, t, r) in shared memory, the column form's registers hold fewer sites.
 inline long long oc_most_systems(long long N, bool mixed, int nsm, size_t smem_sm)

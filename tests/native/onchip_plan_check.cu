@@ -74,6 +74,13 @@ int main()
                                           [](const hh::OcPlan &) { return 64; },
                                           [](const hh::OcPlan &) { return false; });
     if (none.ok) return fail("all refused", 1, 32, 64, 2, 64, none.cols);
+    // Phase numbers go up, and the 2^28 of a launch hold no multiple of 2^32.
+    for (unsigned long long last : {0ull, 1ull, 0xeffffffeull, 0xefffffffull, 0xf0000000ull, 0xfffffffeull, 0xffffffffull,
+                                    0x100000000ull, 0x5ffffffffull, 0x600000000ull}) {
+        const unsigned long long first = hh::oc_first_phase(last), end = first + 0x0fffffffull;
+        if (first <= last || (first & 0xffffffffull) == 0 || first >> 32 != end >> 32)
+            return fail("phase number", 0, 0, 0, 0, (int)last, (long long)first);
+    }
     if (layouts < 10000) return fail("layouts", 0, 0, 0, 0, 0, layouts);
     std::printf("ok\n");
     return 0;
