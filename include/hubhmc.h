@@ -328,6 +328,23 @@ int hh_counters_reset(hh_ctx *ctx, int profile_engine);
  * counters are filled all the same). */
 int hh_counters_get(hh_ctx *ctx, hh_counters *out);
 
+/* Which engine solves n_rhs right-hand sides of a context, and how it is laid out. */
+typedef struct {
+    int onchip;             /* 1: the on-chip engine (the CG vectors stay in the GPU's shared
+                               memory and registers); 0: the grid engine, and the fields
+                               up to x_global are 0 */
+    int tiles_o, tiles_tau; /* tiles of a system over x (d = 1) or z (d = 3) and over tau */
+    int threads;            /* threads per block (a block holds one tile) */
+    int blocks_per_sm;      /* blocks one SM holds at most */
+    int slices;             /* column form: time slices per thread; 0: tile form */
+    int x_global;           /* 1: x stays in global memory */
+    long long onchip_launches; /* on-chip launches since the last hh_counters_reset */
+} hh_layout;
+
+/* Fill *out for n_rhs right-hand sides (1 .. max(n_pf, 4)).  Launches nothing.
+ * Errors: HH_EINVAL. */
+int hh_solver_layout(hh_ctx *ctx, int n_rhs, hh_layout *out);
+
 /* ---- Batched multi-chain engine and serving loop ---------------------------
  * Many independent Markov chains and solves, of different lattices, share one
  * persistent CG launch (an extension: the paper's Sec. 5 runs one lattice at

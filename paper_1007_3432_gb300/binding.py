@@ -82,6 +82,15 @@ class hh_counters(ctypes.Structure):
         return {k: getattr(self, k) for k, _ in self._fields_}
 
 
+class hh_layout(ctypes.Structure):
+    _fields_ = [("onchip", ctypes.c_int), ("tiles_o", ctypes.c_int), ("tiles_tau", ctypes.c_int),
+                ("threads", ctypes.c_int), ("blocks_per_sm", ctypes.c_int), ("slices", ctypes.c_int),
+                ("x_global", ctypes.c_int), ("onchip_launches", ctypes.c_longlong)]
+
+    def as_dict(self):
+        return {k: getattr(self, k) for k, _ in self._fields_}
+
+
 class hh_request(ctypes.Structure):
     _fields_ = [("kind", ctypes.c_int), ("lat", hh_lattice), ("prm", hh_params),
                 ("sigma", ctypes.c_void_p), ("b", ctypes.c_void_p), ("out", ctypes.c_void_p),
@@ -184,6 +193,7 @@ def load(path: str = None):
         "hh_batch_set_timeout": (i, [vp, d]),
         "hh_counters_reset": (i, [vp, i]),
         "hh_counters_get": (i, [vp, ctypes.POINTER(hh_counters)]),
+        "hh_solver_layout": (i, [vp, i, ctypes.POINTER(hh_layout)]),
         "hh_bounds_check": (i, [i, ctypes.POINTER(i), ctypes.POINTER(ctypes.c_longlong)]),
         "hh_solve_noalloc": (i, [ctypes.POINTER(hh_lattice), ctypes.POINTER(hh_params), vp, vp, vp, vp,
                                  ctypes.POINTER(hh_solve_info)]),
@@ -422,6 +432,12 @@ class Context:
         c = hh_counters()
         check(self._lib.hh_counters_get(self._h, ctypes.byref(c)), "hh_counters_get")
         return c.as_dict()
+
+    def solver_layout(self, n_rhs):
+        """Engine and layout of a solve of n_rhs right-hand sides (hh_solver_layout)."""
+        out = hh_layout()
+        check(self._lib.hh_solver_layout(self._h, n_rhs, ctypes.byref(out)), "hh_solver_layout")
+        return out.as_dict()
 
 
 def bounds_check(selftest=False):

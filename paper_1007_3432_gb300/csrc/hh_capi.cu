@@ -190,7 +190,7 @@ struct hh_ctx {
     int smem_sm, smem_blk;
     EngTotals *d_totals;
     // counters and optional CUDA-event profile of the engine launches
-    long long n_launch, n_engine;
+    long long n_launch, n_engine, n_onchip;
     int profile;
     int ev_cap, ev_used;
     cudaEvent_t *ev;
@@ -300,10 +300,9 @@ bool oc_alloc(hh_ctx *c)
 }
 
 // Layout of the on-chip engine for n_rhs systems; ok = 0: the grid engine solves them.
-OcPlan ctx_oc_plan(hh_ctx *c, int n_rhs)
+OcPlan ctx_oc_layout(hh_ctx *c, int n_rhs)
 {
-    OcPlan none = {};
-    if (n_rhs > c->oc_cap) return none;
+    if (n_rhs > c->oc_cap) return OcPlan{};
     if (!c->oc_known[n_rhs]) {
         const bool mixed = c->prm.precision != HH_FP64;
         c->oc_plans[n_rhs] = oc_plan(c->lat.d, c->lat.nx, c->lat.ntau, n_rhs, mixed, c->prm.cheb_degree > 0,
@@ -311,11 +310,16 @@ OcPlan ctx_oc_plan(hh_ctx *c, int n_rhs)
                                      (size_t)c->smem_sm, (size_t)c->smem_blk, c->oc_forms);
         c->oc_known[n_rhs] = true;
     }
-    const OcPlan &p = c->oc_plans[n_rhs];
-    if (!p.ok) return none;
+    return c->oc_plans[n_rhs];
+}
+
+// The layout of the next solve, its packets cleared when the last one had another.
+OcPlan ctx_oc_plan(hh_ctx *c, int n_rhs)
+{
+    const OcPlan p = ctx_oc_layout(c, n_rhs);
     // Other tiles publish other sites: forget the packets of the last layout.
-    if (c->oc_last != n_rhs) {
-        if (cudaMemsetAsync(c->d_pkt, 0, oc_packets(c, c->oc_cap), c->stream) != cudaSuccess) return none;
+    if (p.ok && c->oc_last != n_rhs) {
+        if (cudaMemsetAsync(c->d_pkt, 0, oc_packets(c, c->oc_cap), c->stream) != cudaSuccess) return OcPlan{};
         c->oc_last = n_rhs;
     }
     return p;
@@ -468,6 +472,7 @@ int run_engine(hh_ctx *c)
         O.max_iters = (2LL * c->prm.cheb_degree + 1) * (3LL * (long long)c->prm.cg_maxit + 64);
         HH_TRY(oc_launch(O, P.oc, c->lat.d, c->stream));
         c->n_launch += 1;
+        c->n_onchip += 1;
     }
     EngLaunch L;
     L.sys = c->d_sys;
@@ -1245,6 +1250,7 @@ int hh_counters_reset(hh_ctx *c, int profile_engine)
     HH_TRY(cudaStreamSynchronize(c->stream));
     c->n_launch = 0;
     c->n_engine = 0;
+    c->n_onchip = 0;
     c->ev_used = 0;
     c->profile = profile_engine ? 1 : 0;
     if (c->profile && !c->ev) {
@@ -1285,6 +1291,25 @@ int hh_counters_get(hh_ctx *c, hh_counters *out)
     out->fp64_steps = t.fp64_steps;
     out->sites = c->N;
     return aerr ? aerr : HH_OK;
+}
+
+int hh_solver_layout(hh_ctx *c, int n_rhs, hh_layout *out)
+{
+    if (!c || !out) return HH_EINVAL;
+    const int rc = ensure_rhs(c, n_rhs);
+    if (rc) return rc;
+    memset(out, 0, sizeof(*out));
+    out->onchip_launches = c->n_onchip;
+    const OcPlan p = ctx_oc_layout(c, n_rhs);
+    if (!p.ok) return HH_OK;
+    out->onchip = 1;
+    out->tiles_o = p.go;
+    out->tiles_tau = p.gt;
+    out->threads = p.threads;
+    out->blocks_per_sm = (p.go * p.gt * n_rhs + c->nsm - 1) / c->nsm;
+    out->slices = p.cols;
+    out->x_global = p.x_global;
+    return HH_OK;
 }
 
 }  // extern "C"

@@ -45,3 +45,25 @@ def test_group_sweep_equals_single_applies(hh, d, nx, ntau, dtype, op, k):
                 assert torch.allclose(y[v], yv, rtol=1e-5, atol=1e-5)
             else:
                 assert torch.equal(y[v], yv), v
+
+
+@pytest.mark.parametrize("dtype,d,nx,ntau,k", [(torch.float64, 1, 1000, 900, 4), (torch.float64, 3, 21, 96, 4),
+                                               (torch.float32, 1, 2000, 900, 5), (torch.float32, 3, 22, 180, 3)])
+def test_group_sized_by_the_l2(hh, dtype, d, nx, ntau, k):
+    """Lattices on which half of the L2 (x, t and y of 64 MiB), not the CG
+    scratch, sets the group: two or three vectors, and a remainder."""
+    n = nx ** d * ntau
+    esz = 4 if dtype == torch.float32 else 8
+    group = (64 << 20) // (3 * n * esz)
+    assert 2 <= group < k <= 4 * 8 // esz and k % group != 0
+    x = torch.from_numpy(np.stack([workloads.source(n, seed=73, rhs=a) for a in range(k)])).to(dtype).cuda()
+    with hh.Context(d, nx, ntau) as ctx:
+        ctx.set_field(torch.from_numpy(workloads.sigma_field(n, seed=74)).cuda())
+        y = torch.full_like(x, float("nan"))
+        ctx.counters_reset()
+        ctx.apply_multi(hh.HH_OP_MTM, x, y, k)
+        assert ctx.counters()["kernel_launches"] == 2 * ((k + group - 1) // group)
+        for v in range(k):
+            xv, yv = x[v].clone(), torch.empty_like(x[v])
+            ctx.apply(hh.HH_OP_MTM, xv, yv)
+            assert torch.equal(y[v], yv), v

@@ -43,17 +43,20 @@ def _check_solution(d, nx, ntau, sigma, b, x):
         assert np.linalg.norm(res) <= 1.0001e-10 * np.linalg.norm(b[a])
 
 
-# (precision, Nx, Ntau): 98k-site systems share the grid in the flat engine
-# form; 332k-site FP64 systems are each tiled over the whole grid, with the
-# control warp (overlapped layout).
-@pytest.mark.parametrize("precision,nx,ntau", [("fp64", 16, 24), ("mixed", 16, 24), ("fp64", 24, 24)])
-def test_engine_wait_runs_out_then_context_recovers(hh, monkeypatch, precision, nx, ntau):
+# (precision, Nx, Ntau, on-chip).  98k-site systems: in the on-chip engine (FP64 column
+# or tile form, FP32), or sharing the grid in the grid engine's flat form.  332k-site
+# FP64 systems: each tiled over the whole grid, with the control warp (overlapped layout).
+@pytest.mark.parametrize("precision,nx,ntau,onchip", [("fp64", 16, 24, 1), ("fp64", 10, 24, 1), ("mixed", 16, 24, 1),
+                                                      ("fp64", 16, 24, 0), ("mixed", 16, 24, 0), ("fp64", 24, 24, 0)])
+def test_engine_wait_runs_out_then_context_recovers(hh, monkeypatch, precision, nx, ntau, onchip):
     from paper_1007_3432_gb300.binding import HH_ETIMEOUT
     d = 3
     n = nx ** d * ntau
     sigma = workloads.sigma_field(n, seed=901)
     b = np.stack([workloads.source(n, seed=902, rhs=a) for a in range(2)])
+    monkeypatch.setenv("HH_ENGINE_ONCHIP", str(onchip))
     with hh.Context(d, nx, ntau, precision=precision) as ctx:
+        assert ctx.solver_layout(2)["onchip"] == onchip
         ctx.set_field(torch.from_numpy(sigma).cuda())
         b_d = torch.from_numpy(b).cuda()
         x = torch.zeros_like(b_d)

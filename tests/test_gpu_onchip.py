@@ -44,7 +44,11 @@ def _solve(hh, monkeypatch, onchip, d, nx, ntau, precision, b, sigma, x0=None, *
         x = torch.full(b.shape, 3.0, dtype=torch.float64, device="cuda") if x0 is None else dev(x0.copy())
         ctx.counters_reset()
         rc, info = ctx.solve(dev(b), x, b.shape[0], guess=x0 is not None, allow=(hh.binding.HH_ENOCONV,))
-        return rc, info, x.cpu().numpy(), ctx.counters()
+        cnt = ctx.counters()
+        cnt["layout"] = ctx.solver_layout(b.shape[0])
+        # which engine ran: no silent fall-back to the other
+        assert cnt["layout"]["onchip_launches"] == cnt["layout"]["onchip"] <= (onchip != 0), cnt
+        return rc, info, x.cpu().numpy(), cnt
 
 
 SHAPES = [(1, 2, 2), (1, 2, 7), (1, 3, 2), (1, 17, 5), (1, 33, 40), (1, 300, 11), (1, 731, 24), (3, 2, 2), (3, 2, 9),
@@ -64,30 +68,46 @@ def test_onchip_solve_matches_oracle_and_grid_engine(hh, monkeypatch, d, nx, nta
     kw = dict(cheb_degree=cheb, cheb_eps=1e-3)
     rc, info, x, cnt = _solve(hh, monkeypatch, form, d, nx, ntau, precision, b, sigma, **kw)
     rc0, info0, x0, cnt0 = _solve(hh, monkeypatch, 0, d, nx, ntau, precision, b, sigma, **kw)
+    lay = cnt["layout"]
+    if form == 3 and (d, nx, ntau, n_rhs) == (3, 16, 17, 4):
+        assert lay["onchip"] == 0
+        pytest.skip("no column layout: 16 planes of 256 sites in 17 slices, four times, need two rows per block")
+    assert lay["onchip"] == 1 and (form == 1 or (lay["slices"] > 0) == (form == 3)), lay
     # a mixed on-chip solve is one launch more (the grid engine, for a hand-over)
-    assert form == 3 or precision == "fp64" or cnt["kernel_launches"] == cnt0["kernel_launches"] + 1
+    assert cnt["kernel_launches"] == cnt0["kernel_launches"] + (1 if precision == "mixed" else 0)
     assert rc == 0 and rc0 == 0 and info["converged"] == 1 and info["true_relres"] <= 1e-10
     lat = oracle.lattice(d, nx, ntau)
     L = oracle.links(lat, A, sigma)
     for a in range(n_rhs):
-        res = b[a] - oracle.apply_MTM(lat, H, L, x[a])
-        assert np.linalg.norm(res) <= 1.0001e-10 * np.linalg.norm(b[a])
+        for sol in (x, x0):
+            res = b[a] - oracle.apply_MTM(lat, H, L, sol[a])
+            assert np.linalg.norm(res) <= 1.0001e-10 * np.linalg.norm(b[a])
     assert abs(info["iterations"] - info0["iterations"]) <= 2 + 0.03 * info0["iterations"], (info, info0)
     assert np.linalg.norm(x - x0) <= 1e-4 * np.linalg.norm(x0)
     assert cnt["solves"] == n_rhs and cnt["cg_steps"] > 0
 
 
-@pytest.mark.parametrize("d,nx,ntau,precision,n_rhs", [(3, 16, 64, "fp64", 2), (1, 1024, 160, "fp64", 2),
-                                                       (3, 20, 96, "mixed", 1), (1, 2048, 96, "mixed", 3)])
-def test_onchip_large_lattices(hh, monkeypatch, d, nx, ntau, precision, n_rhs):
-    """Tiles of hundreds to thousands of sites, two and more blocks per SM, x
-    in global memory: capped at 60 steps, where both engines hold the same
-    iterate up to rounding (FP64: 1e-10; FP32 steps between reliable updates:
-    1e-4 of the iterate)."""
+# (lattice, right-hand sides, blocks per SM, x in global memory, column form)
+LARGE = [(3, 16, 64, "fp64", 2, 1, 1, False), (1, 1024, 160, "fp64", 2, 1, 0, False),
+         (3, 17, 33, "fp64", 1, 2, 0, False), (3, 22, 27, "fp64", 1, 2, 1, False),
+         (3, 14, 84, "fp64", 2, 2, 1, False), (1, 136, 151, "fp64", 4, 2, 0, True),
+         (3, 20, 96, "mixed", 1, 1, 0, False), (1, 2048, 96, "mixed", 3, 1, 0, False),
+         (3, 21, 108, "mixed", 1, 1, 1, False), (3, 22, 39, "mixed", 2, 2, 1, False),
+         (1, 557, 103, "mixed", 3, 2, 0, True), (3, 8, 157, "mixed", 2, 2, 0, True)]
+
+
+@pytest.mark.parametrize("d,nx,ntau,precision,n_rhs,per_sm,x_global,column", LARGE)
+def test_onchip_large_lattices(hh, monkeypatch, d, nx, ntau, precision, n_rhs, per_sm, x_global, column):
+    """Tiles of hundreds to thousands of sites, one and two blocks per SM, x
+    in shared and in global memory, in both forms: capped at 60 steps, where
+    both engines hold the same iterate up to rounding (FP64: 1e-10; FP32 steps
+    between reliable updates: 1e-4 of the iterate)."""
     n = nx ** d * ntau
     sigma = workloads.sigma_field(n, seed=1600 + nx)
     b = np.stack([workloads.source(n, seed=1601, rhs=a) for a in range(n_rhs)])
-    rc, info, x, _ = _solve(hh, monkeypatch, 1, d, nx, ntau, precision, b, sigma, cg_maxit=60)
+    rc, info, x, cnt = _solve(hh, monkeypatch, 1, d, nx, ntau, precision, b, sigma, cg_maxit=60)
+    lay = cnt["layout"]
+    assert (lay["onchip"], lay["blocks_per_sm"], lay["x_global"], lay["slices"] > 0) == (1, per_sm, x_global, column), lay
     rc0, info0, x0, _ = _solve(hh, monkeypatch, 0, d, nx, ntau, precision, b, sigma, cg_maxit=60)
     assert rc == rc0 == hh.binding.HH_ENOCONV and info["iterations"] == info0["iterations"] == 60
     tol = 1e-10 if precision == "fp64" else 1e-4
@@ -103,7 +123,8 @@ def test_onchip_guess_and_zero_source(hh, monkeypatch, precision, form):
     sigma = workloads.sigma_field(n, seed=1700)
     b = np.stack([workloads.source(n, seed=1701, rhs=a) for a in range(2)])
     b[1] = 0.0
-    rc, info, x, _ = _solve(hh, monkeypatch, form, d, nx, ntau, precision, b, sigma)
+    rc, info, x, cnt = _solve(hh, monkeypatch, form, d, nx, ntau, precision, b, sigma)
+    assert cnt["layout"]["onchip"] == 1
     assert rc == 0 and not np.any(x[1]) and info["true_relres"] <= 1e-10
     x0 = x * (1.0 + 1e-6)
     x0[1] = 5.0                      # dropped: b = 0 has the solution 0
@@ -113,24 +134,29 @@ def test_onchip_guess_and_zero_source(hh, monkeypatch, precision, form):
     assert np.linalg.norm(x2[0] - x[0]) <= 1e-4 * np.linalg.norm(x[0])
 
 
-@pytest.mark.parametrize("form", [2, 3])
+@pytest.mark.parametrize("form,order", [(2, 0), (3, 0), (1, 1)])
 @pytest.mark.parametrize("d,nx,ntau", [(1, 48, 64), (3, 6, 16)])
-def test_onchip_mixed_hands_over_to_fp64_steps(hh, monkeypatch, d, nx, ntau, form):
+def test_onchip_mixed_hands_over_to_fp64_steps(hh, monkeypatch, d, nx, ntau, form, order):
     """With reliable_delta = 0.9 each reliable update follows a drop of 10%,
     which counts as a stall: after two the systems go on with FP64 steps, in
-    the grid engine, from the on-chip state."""
+    the grid engine, from the on-chip state (of both forms, and of the
+    exact-block form of M)."""
     n = nx ** d * ntau
     sigma = workloads.sigma_field(n, seed=1800)
     b = np.stack([workloads.source(n, seed=1801, rhs=a) for a in range(2)])
     b[1] = 0.0                       # done on the chip; the other goes on
-    rc, info, x, cnt = _solve(hh, monkeypatch, form, d, nx, ntau, "mixed", b, sigma, reliable_delta=0.9)
-    rc0, info0, x0, cnt0 = _solve(hh, monkeypatch, 0, d, nx, ntau, "mixed", b, sigma, reliable_delta=0.9)
+    rc, info, x, cnt = _solve(hh, monkeypatch, form, d, nx, ntau, "mixed", b, sigma, reliable_delta=0.9,
+                               link_order=order)
+    rc0, info0, x0, cnt0 = _solve(hh, monkeypatch, 0, d, nx, ntau, "mixed", b, sigma, reliable_delta=0.9,
+                               link_order=order)
+    assert cnt["layout"]["onchip"] == 1 and cnt0["layout"]["onchip"] == 0
     assert cnt["fp64_steps"] > 0 and cnt0["fp64_steps"] > 0, (cnt, cnt0)
     assert abs(cnt["cg_steps"] - cnt0["cg_steps"]) <= 2 + 0.03 * cnt0["cg_steps"]
     assert rc == 0 and info["converged"] == 1 and info["true_relres"] <= 1e-10 and not np.any(x[1])
     lat = oracle.lattice(d, nx, ntau)
     L = oracle.links(lat, A, sigma)
-    res = b[0] - oracle.apply_MTM(lat, H, L, x[0])
+    q = oracle.apply_MTM_ex(lat, H, L, 1, x[0]) if order else oracle.apply_MTM(lat, H, L, x[0])
+    res = b[0] - q
     assert np.linalg.norm(res) <= 1.0001e-10 * np.linalg.norm(b[0])
 
 
@@ -145,7 +171,9 @@ def test_onchip_layouts_alternate_in_one_context(hh, monkeypatch):
 
     def one(ctx, k):
         x = torch.zeros(k, n, dtype=torch.float64, device="cuda")
+        ctx.counters_reset()
         ctx.solve(b[:k].clone(), x, k)
+        assert ctx.solver_layout(k)["onchip_launches"] == 1
         return x.cpu()
 
     fresh = {}
@@ -171,6 +199,7 @@ def test_onchip_exact_block_first_order(hh, monkeypatch, d, nx, ntau, precision,
     b = np.stack([workloads.source(n, seed=2001, rhs=a) for a in range(n_rhs)])
     rc, info, x, cnt = _solve(hh, monkeypatch, 1, d, nx, ntau, precision, b, sigma, link_order=1)
     rc0, info0, x0, _ = _solve(hh, monkeypatch, 0, d, nx, ntau, precision, b, sigma, link_order=1)
+    assert cnt["layout"]["onchip"] == 1
     assert rc == 0 and rc0 == 0 and info["converged"] == 1 and info["true_relres"] <= 1e-10
     lat = oracle.lattice(d, nx, ntau)
     L = oracle.links(lat, A, sigma)
@@ -195,6 +224,7 @@ def test_onchip_solve_replays_from_a_graph(hh, monkeypatch, precision):
         with hh.Context(d, nx, ntau, precision=precision) as ctx:
             ctx.set_field(dev(workloads.sigma_field(n, seed=2101)))
             ctx.solve(b, x, 1)
+            assert ctx.solver_layout(1)["onchip_launches"] == 1
             ref = x.clone()
             stream.synchronize()
             g = torch.cuda.CUDAGraph()
@@ -236,6 +266,7 @@ def test_captured_solve_replays_after_other_solves(hh, monkeypatch, onchip, prec
             g = torch.cuda.CUDAGraph()
             with torch.cuda.graph(g, stream=stream):
                 ctx.solve(b[:2], xa, 2, info=False)
+            assert ctx.solver_layout(2)["onchip_launches"] == onchip
             for guess in (False, True):
                 xa.zero_()
                 g.replay()
