@@ -86,12 +86,12 @@ def bytes_per_site(kind, precision):
     return 4 * 8 + (12 if precision != "fp64" else 0)
 
 
-# DRAM bytes per engine iteration (two right-hand sides) of the engine kernel
-# as it stands, from one ncu --set full capture each (dram__bytes_read.sum +
+# DRAM bytes per iteration (two right-hand sides) of the grid engine as it
+# stands, from one ncu --set full capture each (dram__bytes_read.sum +
 # dram__bytes_write.sum over a 202-iteration launch; profiles/engine_kernel_*).
-# A launch's traffic scales with its iterations.
-ENGINE_DRAM_PER_ITER = {("d1_nx1024_nt512", "fp64"): (12724992 + 70935296) / 202.0,
-                        ("d3_nx32_nt128", "mixed"): (35195983000 + 27069706000) / 202.0}
+# A launch's traffic scales with its iterations.  On the chip the vectors of a
+# solve do not cross HBM.
+ENGINE_DRAM_PER_ITER = {("d3_nx32_nt128", "mixed"): (35195983000 + 27069706000) / 202.0}
 
 # DRAM bytes (read + write) per launch of the Q apply from one ncu capture each
 # (profiles/mtm_*): (workload, dtype, vectors per launch) -> bytes.
@@ -99,15 +99,51 @@ APPLY_DRAM_PER_LAUNCH = {("d3_nx32_nt128", "fp32", 1): 33557760 + 344320 + 88320
                          ("d3_nx32_nt128", "fp32", 16): 300300288 + 229754880}
 
 
-def engine_traffic(wl, precision, cheb, cnt):
+def engine_traffic(wl, precision, cheb, cnt, layout):
     """Estimated DRAM bytes per engine launch, or None without a capture."""
     per_iter = ENGINE_DRAM_PER_ITER.get((wl.name, precision))
-    if per_iter is None or cheb or cnt["engine_launches"] == 0:
+    if per_iter is None or cheb or layout["onchip"] or cnt["engine_launches"] == 0:
         return None
     # both right-hand sides advance together: one INIT iteration, then the CG
     # steps and true-residual checks of one system
     iters = (cnt["cg_steps"] + cnt["ru_steps"]) / 2.0 / cnt["engine_launches"] + 1.0
     return per_iter * iters
+
+
+def engine_roofline(wl, precision, cheb, cnt, layout):
+    """Roofline of the CG solves: in FP64 the operations against the FP64 peak;
+    in mixed precision the algorithmic bytes against HBM, or, when the solves
+    run on the chip and their vectors do not cross HBM, the operations of the
+    FP32 steps (the FP64 reliable updates, a few in a thousand, counted with
+    them) against the FP32 peak.  With the Chebyshev preconditioner every CG
+    step and true-residual check is followed by 2n sub-steps, each one Q apply
+    with its vector update (counted at the flops of a CG step)."""
+    peaks, src = measured_peaks()
+    n = wl.nsites
+    eng_s = cnt["engine_ms"] / 1000.0
+    f_cg, f_ru = flops_per_site(wl.d, "cg", precision), flops_per_site(wl.d, "ru", precision)
+    flops = n * (cnt["cg_steps"] * f_cg + cnt["ru_steps"] * f_ru)
+    flops += n * (cnt["cg_steps"] + cnt["ru_steps"]) * 2 * cheb * f_cg
+    onchip = bool(layout["onchip"])
+    kernel = ("on-chip engine, %s" % ("column form (k_onchip_cols)" if layout["slices"] else "tile form (k_onchip)")
+              if onchip else "grid engine (engine_kernel)")
+    kernel += ", FP64 CG" if precision == "fp64" else ", FP32-inner CG"
+    out = {"traffic": engine_traffic(wl, precision, cheb, cnt, layout), "kernel": kernel}
+    if precision == "fp64" or onchip:
+        fp64 = precision == "fp64"
+        peak = fp64_peak_tflops() if fp64 else fp32_peak_tflops()
+        ach = flops / eng_s / 1e12 if eng_s > 0 else 0.0
+        out.update(bound="alu", achieved=ach, peak=peak, unit="TFLOP/s", frac=ach / peak,
+                   peak_source="%s from unit counts and clocks (152 SMs x %s x 2.07 GHz)"
+                               % (("FP64", "2 DFMA/clk") if fp64 else ("FP32", "128 FFMA/clk")))
+    else:
+        byts = n * (cnt["cg_steps"] * bytes_per_site("cg", precision)
+                    + cnt["ru_steps"] * bytes_per_site("ru", precision))
+        ach = byts / eng_s / 1e9 if eng_s > 0 else 0.0
+        out.update(bound="hbm", achieved=ach, peak=peaks["hbm_gbs"], unit="GB/s", frac=ach / peaks["hbm_gbs"],
+                   peak_source="%s MEASURED_PEAKS.json hbm_gbs" % src,
+                   algorithmic_bytes_per_site_cg_step=bytes_per_site("cg", precision))
+    return out
 
 
 def us_per_engine_iteration(cnt, n_rhs=2):
@@ -123,6 +159,12 @@ def fp64_peak_tflops():
     clock per SM x 2 flops x 2.07 GHz (maximum SM clock) = 1.26 TFLOP/s, the
     nominal 1.25 TFLOP/s of the part."""
     return 152 * 2 * 2 * 2.07e9 / 1e12
+
+
+def fp32_peak_tflops():
+    """FP32 peak from unit counts and clocks: 152 SMs x 128 FFMA per clock x 2
+    flops x 2.07 GHz."""
+    return 152 * 128 * 2 * 2.07e9 / 1e12
 
 
 def measured_peaks():
@@ -369,30 +411,9 @@ def measure_solve(wl, precision, rank, dev, stream, steps, warmup, flush, cg_max
         dev_ms.append(a)
         wall_ms.append(w)
     cnt = ctx.counters()
+    roof = engine_roofline(wl, precision, cheb, cnt, ctx.solver_layout(2))
     ctx.close()
-    peaks, src = measured_peaks()
-    eng_s = cnt["engine_ms"] / 1000.0
-    # With the Chebyshev preconditioner every CG step and true-residual check
-    # is followed by 2n sub-steps, each one Q apply with its vector update
-    # (counted at the flops of a CG step).
     q_per_step = 2 * cheb + 1
-    if precision == "fp64":
-        flops = n * (cnt["cg_steps"] * flops_per_site(wl.d, "cg", "fp64") + cnt["ru_steps"] * flops_per_site(wl.d, "ru", "fp64"))
-        flops += n * (cnt["cg_steps"] + cnt["ru_steps"]) * (q_per_step - 1) * flops_per_site(wl.d, "cg", "fp64")
-        ach = flops / eng_s / 1e12
-        roof = {"bound": "alu", "achieved": ach, "peak": fp64_peak_tflops(), "unit": "TFLOP/s",
-                "frac": ach / fp64_peak_tflops(), "traffic": engine_traffic(wl, precision, cheb, cnt),
-                "kernel": "engine_kernel (FP64 CG)",
-                "peak_source": "FP64 from unit counts and clocks (152 SMs x 2 DFMA/clk x 2.07 GHz)"}
-    else:
-        byts = n * (cnt["cg_steps"] * bytes_per_site("cg", precision)
-                    + cnt["ru_steps"] * bytes_per_site("ru", precision))
-        ach = byts / eng_s / 1e9
-        roof = {"bound": "hbm", "achieved": ach, "peak": peaks["hbm_gbs"], "unit": "GB/s",
-                "frac": ach / peaks["hbm_gbs"], "traffic": engine_traffic(wl, precision, cheb, cnt),
-                "kernel": "engine_kernel (FP32-inner CG)",
-                "peak_source": "%s MEASURED_PEAKS.json hbm_gbs" % src,
-                "algorithmic_bytes_per_site_cg_step": bytes_per_site("cg", precision)}
     t_dev = sum(dev_ms) / 1000.0
     t_wall = sum(wall_ms) / 1000.0
     return {"workload": wl.name, "precision": precision, "solves": cnt["solves"],
@@ -958,33 +979,9 @@ def main():
     value = tot_applies / t_dev
     e2e = tot_applies / t_wall
 
-    # Roofline of the dominant kernel: the persistent CG engine.
-    f_cg = flops_per_site(wl.d, "cg", args.precision)
-    f_ru = flops_per_site(wl.d, "ru", args.precision)
-    peaks, src = measured_peaks()
-    eng_s = cnt["engine_ms"] / 1000.0
-    per_launch = eng_s / max(1, cnt["engine_launches"])
-    if args.precision == "fp64":
-        flops = n * (cnt["cg_steps"] * f_cg + cnt["ru_steps"] * f_ru)
-        # preconditioner sub-steps: one Q apply with its vector update each,
-        # counted at the flops of a CG step
-        flops += n * (cnt["cg_steps"] + cnt["ru_steps"]) * (q_per_step - 1) * f_cg
-        achieved = flops / eng_s / 1e12 if eng_s > 0 else 0.0
-        peak = fp64_peak_tflops()
-        roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-                "frac": achieved / peak, "traffic": engine_traffic(wl, args.precision, args.cheb, cnt),
-                "kernel": "engine_kernel (persistent FP64 CG)",
-                "peak_source": "FP64 from unit counts and clocks (152 SMs x 2 DFMA/clk x 2.07 GHz)",
-                "launch_ms": per_launch * 1000.0}
-    else:
-        byts = n * (cnt["cg_steps"] * bytes_per_site("cg", args.precision)
-                    + cnt["ru_steps"] * bytes_per_site("ru", args.precision))
-        achieved = byts / eng_s / 1e9 if eng_s > 0 else 0.0
-        peak = peaks["hbm_gbs"]
-        roof = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                "frac": achieved / peak, "traffic": None,
-                "kernel": "engine_kernel (persistent FP32-inner CG)",
-                "peak_source": "%s MEASURED_PEAKS.json hbm_gbs" % src, "launch_ms": per_launch * 1000.0}
+    # Roofline of the dominant kernel: the CG engine.
+    roof = engine_roofline(wl, args.precision, args.cheb, cnt, ctx.solver_layout(2))
+    roof["launch_ms"] = cnt["engine_ms"] / max(1, cnt["engine_launches"])
 
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,

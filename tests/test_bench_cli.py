@@ -99,3 +99,20 @@ def test_us_per_engine_iteration():
     assert abs(bench.us_per_engine_iteration(cnt) - 30090.0 / 1003.0) < 1e-9
     assert bench.us_per_engine_iteration({"cg_steps": 0, "ru_steps": 0, "engine_launches": 0,
                                           "engine_ms": 0.0}) is None
+
+
+def test_roofline_names_the_engine_that_ran():
+    """The roofline's kernel, bound and traffic follow the layout of the
+    solves: on the chip the vectors do not cross HBM."""
+    import bench
+    cnt = {"cg_steps": 2000, "ru_steps": 10, "engine_launches": 1, "engine_ms": 10.0}
+    grid = {"onchip": 0, "slices": 0}
+    tile, cols = {"onchip": 1, "slices": 0}, {"onchip": 1, "slices": 4}
+    r = bench.engine_roofline(bench.WORKLOADS["c1"], "fp64", 0, cnt, tile)
+    assert "k_onchip)" in r["kernel"] and "engine_kernel" not in r["kernel"] and r["traffic"] is None
+    assert r["bound"] == "alu" and r["peak"] == bench.fp64_peak_tflops()
+    r = bench.engine_roofline(bench.WORKLOADS["c0"], "mixed", 0, cnt, cols)
+    assert "k_onchip_cols" in r["kernel"] and r["bound"] == "alu" and r["peak"] == bench.fp32_peak_tflops()
+    r = bench.engine_roofline(bench.WORKLOADS["c2"], "mixed", 0, cnt, grid)
+    assert "engine_kernel" in r["kernel"] and r["bound"] == "hbm" and r["traffic"] > 0
+    assert bench.engine_roofline(bench.WORKLOADS["c2"], "fp64", 0, cnt, grid)["bound"] == "alu"
