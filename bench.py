@@ -128,10 +128,14 @@ def engine_roofline(wl, precision, cheb, cnt, layout):
     kernel = ("on-chip engine, %s" % ("column form (k_onchip_cols)" if layout["slices"] else "tile form (k_onchip)")
               if onchip else "grid engine (engine_kernel)")
     kernel += ", FP64 CG" if precision == "fp64" else ", FP32-inner CG"
+    stalled = cnt["fp64_steps"] / max(1, cnt["cg_steps"]) if precision != "fp64" else 0.0
+    if onchip and stalled > 0.0:
+        kernel += "; %.0f%% of the steps in FP64, in the grid engine (engine_kernel)" % (100.0 * stalled)
     out = {"traffic": engine_traffic(wl, precision, cheb, cnt, layout), "kernel": kernel}
     if precision == "fp64" or onchip:
         fp64 = precision == "fp64"
-        peak = fp64_peak_tflops() if fp64 else fp32_peak_tflops()
+        peak = (fp64_peak_tflops() if fp64 else
+                1.0 / ((1.0 - stalled) / fp32_peak_tflops() + stalled / fp64_peak_tflops()))
         ach = flops / eng_s / 1e12 if eng_s > 0 else 0.0
         out.update(bound="alu", achieved=ach, peak=peak, unit="TFLOP/s", frac=ach / peak,
                    peak_source="%s from unit counts and clocks (152 SMs x %s x 2.07 GHz)"

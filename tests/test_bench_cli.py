@@ -105,7 +105,7 @@ def test_roofline_names_the_engine_that_ran():
     """The roofline's kernel, bound and traffic follow the layout of the
     solves: on the chip the vectors do not cross HBM."""
     import bench
-    cnt = {"cg_steps": 2000, "ru_steps": 10, "engine_launches": 1, "engine_ms": 10.0}
+    cnt = {"cg_steps": 2000, "ru_steps": 10, "engine_launches": 1, "engine_ms": 10.0, "fp64_steps": 0}
     grid = {"onchip": 0, "slices": 0}
     tile, cols = {"onchip": 1, "slices": 0}, {"onchip": 1, "slices": 4}
     r = bench.engine_roofline(bench.WORKLOADS["c1"], "fp64", 0, cnt, tile)
@@ -113,6 +113,10 @@ def test_roofline_names_the_engine_that_ran():
     assert r["bound"] == "alu" and r["peak"] == bench.fp64_peak_tflops()
     r = bench.engine_roofline(bench.WORKLOADS["c0"], "mixed", 0, cnt, cols)
     assert "k_onchip_cols" in r["kernel"] and r["bound"] == "alu" and r["peak"] == bench.fp32_peak_tflops()
+    # half of the steps after a stall, in FP64 on the grid engine
+    r = bench.engine_roofline(bench.WORKLOADS["c0"], "mixed", 0, dict(cnt, fp64_steps=1000), cols)
+    assert "50% of the steps in FP64" in r["kernel"]
+    assert abs(r["peak"] - 2.0 / (1.0 / bench.fp32_peak_tflops() + 1.0 / bench.fp64_peak_tflops())) < 1e-9
     r = bench.engine_roofline(bench.WORKLOADS["c2"], "mixed", 0, cnt, grid)
     assert "engine_kernel" in r["kernel"] and r["bound"] == "hbm" and r["traffic"] > 0
     assert bench.engine_roofline(bench.WORKLOADS["c2"], "fp64", 0, cnt, grid)["bound"] == "alu"
