@@ -197,13 +197,28 @@ __device__ __forceinline__ unsigned long long warp_join(unsigned long long x, in
 }
 
 // Sum over the warp, the same in every lane.
-template <typename T>
-__device__ __forceinline__ ISum warp_isum(T v)
+__device__ __forceinline__ ISum warp_isum(double v)
 {
     const Significand p = significand(v);
     ISum r;
     r.e = (int)__reduce_max_sync(0xffffffffu, (unsigned)p.e);
     r.s = warp_join(shift_round(p.m << kGuardWarp, r.e - p.e), 0);
+    return r;
+}
+
+// FP32 values: 24 bits in a window of 54, two parts of 27.  A value within 2^-30 of the
+// largest is added exactly (an FP64 tree adds exactly within 2^-24); one below loses at
+// most 2^-54 of the largest, 16 2^-53 of the sum for a whole warp, where each value
+// carries an FP32 rounding of 2^-24 itself.
+__device__ __forceinline__ ISum warp_isum(float v)
+{
+    const Significand p = significand(v);
+    ISum r;
+    r.e = (int)__reduce_max_sync(0xffffffffu, (unsigned)p.e);
+    const unsigned long long x = shift_round(p.m << 1, r.e - p.e);
+    const unsigned long long hi = __reduce_add_sync(0xffffffffu, (unsigned)(x >> 27));
+    const unsigned long long lo = __reduce_add_sync(0xffffffffu, (unsigned)x & 0x7ffffffu);
+    r.s = ((hi << 27) + lo) << (kGuardWarp - 1);
     return r;
 }
 
