@@ -216,7 +216,10 @@ int hh_apply(hh_ctx *ctx, int op, const void *x, void *y, int dtype);
 int hh_apply_multi(hh_ctx *ctx, int op, const void *x, void *y, int n_vec, int dtype);
 
 /* Solve Q x_a = b_a for a = 0..n_rhs-1 by CG with x0 = 0 (Sec. 4.1) in the
- * context's precision, all right-hand sides in one persistent launch.  With
+ * context's precision, all right-hand sides in one persistent launch: of the
+ * on-chip engine when they fit (hh_solver_layout), else of the grid engine.  In
+ * HH_MIXED an on-chip launch is followed by a grid engine launch, which goes on
+ * with the systems that need FP64 steps and else leaves at once.  With
  * cheb_degree = n > 0 the CG is preconditioned by the Chebyshev polynomial
  * P(Q) of Sec. 4.2, applied as n real quadratic factors (2n applications of
  * Q per step); info->iterations then counts preconditioned steps.
@@ -294,7 +297,7 @@ int hh_leapfrog(hh_ctx *ctx, double *pi, const double *chi, int n_rhs, int n_md,
                 hh_solve_info *info);
 
 /* Bound, in seconds, of every device-side wait of the context's kernels (the
- * persistent CG engine's waits for other blocks' partial sums, the
+ * persistent CG engines' waits for other blocks' partial sums and halos, the
  * multi-vector apply's waits for its bulk copies); default 5.  A wait that
  * runs out makes the kernel record HH_ETIMEOUT and leave: hh_solve and the
  * calls built on it return HH_ETIMEOUT, an apply reports it at the next

@@ -29,10 +29,14 @@
 // What bounds it: the chain exchange - barrier - phase - block sum, run by a few
 // warps (FP64 from about 800 sites per SM: the FP64 pipe, 16 clocks per warp
 // instruction).  Measured against the grid engine, us per iteration: d = 1
-// 1024 x 128 FP64, 2 right-hand sides, 10.5 (15.4), a degree-8 preconditioned
-// step on 256 x 256 89 (199); d = 3 16^3 x 64 mixed, one, 6.9 (15.1), two, 7.7
-// (16.5), 20^3 x 96 mixed, one, 10.5 (18.2).  It was faster wherever the vectors
-// fit (20^3 x 64 mixed, two: 13.7 against 19.4).  Tiles whose column fits a
+// 1024 x 128 FP64, 2 right-hand sides, 10.8 (15.6), 1024 x 512 29.3 (30.1), mixed 9.1
+// (14.3), a degree-8 preconditioned step on 256 x 256 90 (197); d = 3 16^3 x 64
+// mixed, one, 6.7 (15.1), two, 7.6 (16.5), 20^3 x 96 mixed, one, 10.4 (18.0).  It was
+// faster on all of 800 lattices with 1 to 8 right-hand sides drawn among those that fit
+// (4^3 to 24^3, chains of 16 to 2048 sites): by 1.1 at least (14^3 x 99 FP64, two:
+// 29.8 against 32.8), at the median by 2.1 in FP64, 2.7 mixed, 3.2 preconditioned and
+// 2.9 to 3.7 in the exact-block form; whole solves of the smallest (2 x 2 and up) by
+// 1.6 to 3.8.  So a lattice that fits runs here.  Tiles whose column fits a
 // thread's registers run in hh_onchip_cols.cu.
 //
 // Every wait is bounded (EngCtl::timeout_ns); on expiry the block records

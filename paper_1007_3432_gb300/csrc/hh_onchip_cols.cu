@@ -3,7 +3,7 @@
 // The engine of hh_onchip.cu with the same tiles, packets and sums, for tiles
 // whose row of spatial sites is at most one block wide: a thread owns one
 // spatial site and its K time slices (at most) of the tile, and keeps r, p, t,
-// x and the links of that column in registers.  The time neighbours of a site
+// x and the links of that column in registers (but for some spills, below).  The time neighbours of a site
 // are then in the same thread, the row before the tile and the one after it
 // are read from their packets straight into registers, and shared memory only
 // carries the 2d spatial neighbours, at constant strides.  The threads at the
@@ -12,18 +12,24 @@
 // publish; the other warps hand it their partial sums at a barrier they do not
 // wait on.
 //
-// Why: the shared-memory form executes about 300 instructions per site and
-// iteration (index arithmetic, edge tests, addresses), this one about 90, and
-// with a few warps per SM each instruction is 4-8 clocks of the chain exchange -
-// barrier - phase - sum that bounds it.  Measured, us per iteration, two
+// Why: with a few warps per SM each instruction is 4-8 clocks of the chain exchange -
+// barrier - phase - sum that bounds it, and the index arithmetic, edge tests and
+// addresses of the shared-memory form are most of its instructions.  Counted over
+// 200-step solves with two right-hand sides, thread instructions per site and
+// iteration (polls and the control warp included): 12^3 x 64 mixed 164, tile form
+// 479; 8^3 x 40 FP64 380, tile form 962.  Measured, us per iteration, two
 // right-hand sides, against the tile form (and the grid engine): d = 1 32 x 64
-// FP64 4.4, 4.8 (11.3), mixed 3.6, 4.0 (9.6); 731 x 96 mixed 4.4, 5.8 (11.2);
-// 1024 x 128 mixed 5.2, 6.0 (10.7); d = 3 8^3 x 40 FP64 6.3, 7.0 (17.0);
-// 12^3 x 64 mixed 4.8, 7.0 (15.0).  The tile form stays for tiles that do not fit
+// FP64 4.3, 4.8 (11.5), mixed 3.5, 4.3 (9.8); 731 x 96 mixed 4.6, 5.5 (11.3);
+// 1024 x 128 mixed 5.4, 5.9 (10.9); d = 3 8^3 x 40 FP64 6.5, 7.3 (17.1);
+// 12^3 x 64 mixed 4.9, 6.8 (14.7).  The tile form stays for tiles that do not fit
 // (wider rows, more slices than registers) and where it is faster: 16^3 x 64
-// mixed, one right-hand side, 6.9 against 8.5.  The exact-block form of M to first
-// order exists in this form only: observables on 10^3 x 48 FP64, 4 noise vectors,
-// 38.6 ms on the grid engine (scalar loops that recompute the hops), 21.8 here.
+// mixed, one right-hand side, 6.7 against 8.4.  Not all of a column stays in registers:
+// the FP64 kernels of 4 slices spill 16 to 108 bytes a thread (52 to 120 in the
+// exact-block form, 124 to 212 preconditioned), of 8 slices 220 to 284, the preconditioned
+// one of 2 slices with two halo columns 40, and the FP32 ones of 8 slices 8 to 140.  The exact-block form of M to first order exists in this form
+// only, with at most 4 slices: observables on 10^3 x 48 FP64, 4 noise vectors, 38.6 ms
+// on the grid engine (scalar loops that recompute the hops), 22 here; that is the most
+// slices 10^3 can have with 4 vectors.
 #include "hh_onchip_dev.cuh"
 
 namespace hh {

@@ -64,8 +64,11 @@ OcPlan oc_choose(int d, int nx, int ntau, int nsys, bool mixed, bool cheb, bool 
                     // form 0: columns; 1, 2: tile form with x in shared or global memory
                     int K = 0, sides = 1, thr = 0;
                     size_t sm;
-                    // Clocks of one iteration on an SM holding m tiles, from times measured over so,
-                    // st and m on the lattices of the size range (within about 10% of them).
+                    // Clocks of one iteration on an SM holding m tiles, fitted to times over so, st
+                    // and m; what counts is their order.  Times of 500 drawn lattices over this cost,
+                    // median (8 in 10 of them): FP64 columns 1.03 (0.97 - 1.10), tiles 0.94 (0.87 -
+                    // 1.06); mixed columns 1.25 (1.18 - 1.35), tiles 1.26 (1.04 - 1.37).  Of a whole
+                    // preconditioned step (n = 8): columns 10.6 (9.5 - 12.9), tiles 12.7 (10.7 - 15.8).
                     double cost;
                     if (form == 0) {
                         if (!cols_candidate(d, P, nx, go, so, st, mixed, cheb, ex, &K, &sides, &thr)) continue;
