@@ -139,7 +139,8 @@ def engine_roofline(wl, precision, cheb, cnt, layout):
         ach = flops / eng_s / 1e12 if eng_s > 0 else 0.0
         out.update(bound="alu", achieved=ach, peak=peak, unit="TFLOP/s", frac=ach / peak,
                    peak_source="%s from unit counts and clocks (152 SMs x %s x 2.07 GHz)"
-                               % (("FP64", "2 DFMA/clk") if fp64 else ("FP32", "128 FFMA/clk")))
+                               % (("FP64", "2 DFMA/clk") if fp64 else ("FP32", "128 FFMA/clk") if stalled == 0.0 else
+                                  ("FP32 and FP64 steps", "128 FFMA/clk or 2 DFMA/clk")))
     else:
         byts = n * (cnt["cg_steps"] * bytes_per_site("cg", precision)
                     + cnt["ru_steps"] * bytes_per_site("ru", precision))
